@@ -70,3 +70,25 @@ def test_duplicate_removal_matches_oracle(lib):
     assert one[pairs].mean() > 0.9, one[pairs].mean()
     with pytest.raises(mkgb.MkgbError):
         ctx.remove_duplicates(hits, score, np.zeros(seeds.shape[0], np.int32), frac=0.0)
+
+
+@pytest.mark.parametrize("n,width,n_ids", [(1, 1, 4), (257, 3, 40), (600, 5, 90), (700, 22, 2500), (512, 33, 60)])
+def test_items_on_crowded_hits_match_oracle(lib, n, width, n_ids):
+    """Rows on few hits, so that a row meets from none to hundreds of others (more than the kernel
+    keeps in registers), with repeated hits inside a row, empty entries and equal scores."""
+    g, batch, *_ = _duplicate_seed_batch(1, 300)
+    n_hits = batch.hit_xyz.shape[0]
+    assert n_ids <= n_hits
+    rng = np.random.default_rng(n + width)
+    rows = rng.integers(0, n_ids, (n, width)).astype(np.int32)
+    if width > 3:
+        rows[rng.random(rows.shape) < 0.25] = -1
+    score = rng.integers(0, 6, n).astype(np.float32)
+    ctx = pipeline.make_context(g, S.default_params())
+    ctx.load_hits(batch.n_events, batch.hit_off, batch.hit_xyz, batch.hit_cov)
+    for frac in (0.25, 0.5, 1.0):
+        keep = ctx.remove_duplicates(rows, score, np.zeros(n, np.int32), min_hits=width // 4, frac=frac)
+        ref = oracle.remove_duplicates(rows, score.astype(np.float64), n_hits, min_hits=width // 4, frac=frac)
+        assert np.array_equal(keep, ref)
+    if width == 3:
+        assert np.array_equal(ctx.clean_seeds(rows, np.zeros(n, np.int32)), oracle.clean_seeds(rows, n_hits))
