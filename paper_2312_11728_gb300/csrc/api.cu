@@ -915,13 +915,13 @@ int mkgb_fit_grad(mkgb_ctx* ctx, int n, int max_steps, const int32_t* layers, co
     CK(cudaMemsetAsync(gx, 0, 4 * NL, st));
     float* ck = nullptr;
     if (mode == 0) {   // checkpoints of the reverse sweep: 128 bytes per track and step
-        CK(ensure(ctx->grad_ck, 128 * N * std::max<size_t>(M, 1)));
+        CK(ensure(ctx->grad_ck, fit_grad_scratch_bytes(n, max_steps)));
         ck = (float*)ctx->grad_ck.p;
     }
     CK(launch_fit_grad(st, (const DevGeom*)ctx->geom_d.p, ctx->params, (const float4*)ctx->pay.p, ctx->n_hits, n,
                        max_steps, (const int*)dl, (const int*)dh, (const float*)dp0, (const float*)dc0,
                        (const float*)dal, (const float*)dxs, (float*)xo, (float*)gp, (float*)ga, (float*)gx, (int*)so,
-                       ck, ctx->mod_hits));
+                       ck, ctx->n_sms, ctx->mod_hits));
     CK(copy_back(ctx, chi2_out, xo, 4 * N, on_device));
     CK(copy_back(ctx, d_p0, gp, 24 * N, on_device));
     CK(copy_back(ctx, d_align, ga, 24 * NL, on_device));

@@ -5,14 +5,14 @@
 // h' = h + d_l + w_l x (h - c_l), with c_l the origin for a cylinder and (0, 0, z_l) for a disk;
 // the layer surfaces stay nominal.  The thickness scale multiplies x/X0 of the layer.
 //
-// Both kernels run the FP32 fit step (fit_step below) on dual numbers (dual.cuh) carrying KD
-// directional derivatives, one thread per track.
+// The kernels run the FP32 fit step (fit_step below) on dual numbers (dual.cuh) carrying KD
+// directional derivatives.
 //
-// k_fit_adjoint (reverse sweep, the default): a plain FP32 pass stores the input state of every
-// step (a checkpoint per layer); then, from the last step back to the first, the step is redone
-// from its checkpoint with its 34 inputs (27 state words, 6 alignment, 1 thickness scale) seeded
-// KD at a time, and the adjoint of its output (d total / d output, starting at zero after the
-// last step; the step's own chi2 enters with weight 1) is contracted with the output
+// Reverse sweep (the default): a plain FP32 pass (k_fit_ck) stores the input state of every step (a
+// checkpoint per layer); then (k_fit_adjoint), from the last step back to the first, the step is
+// redone from its checkpoint with its 34 inputs (27 state words, 6 alignment, 1 thickness scale)
+// seeded KD at a time, and the adjoint of its output (d total / d output, starting at zero after
+// the last step; the step's own chi2 enters with weight 1) is contracted with the output
 // derivatives: d total / d input = dchi2_j / d input + lambda . d out / d input.  The state part
 // becomes the adjoint for the previous step, the layer part is summed per layer, and the adjoint
 // at the first step's input is d chi2 / d p0.  Cost ~ L x ceil(34 / KD) dual steps per track.
@@ -40,8 +40,9 @@ __device__ __forceinline__ void load_geom(const DevGeom* __restrict__ gp, DevGeo
 
 __device__ __forceinline__ D seeded(float v, int comp, int base) {
     D r(v);
-    const int k = comp - base;
-    if (k >= 0 && k < KD) r.d[k] = 1.0f;
+#pragma unroll
+    for (int k = 0; k < KD; ++k)
+        if (comp - base == k) r.d[k] = 1.0f;
     return r;
 }
 
@@ -214,105 +215,191 @@ __device__ __forceinline__ void load_ck(const float* __restrict__ p, State& t) {
 // the layer's 6 alignment parameters, its thickness scale.
 constexpr int kStateIn = 27, kStepIn = 34;
 
+// Keys of the reverse sweep's order: steps of the track (the longest first) and how many of them
+// cross disks.
+constexpr int kAdjKeyLen = 64, kAdjKeyDisks = 32, kAdjKeys = kAdjKeyLen * kAdjKeyDisks;
+
+// Plain pass of the reverse sweep: one thread per track, the input of every step checkpointed.
 template <bool MOD>
-__global__ void __launch_bounds__(kThreads) k_fit_adjoint(
+__global__ void __launch_bounds__(kThreads) k_fit_ck(
     const DevGeom* __restrict__ gp, DevParams P, const float4* __restrict__ pay, int64_t n_hits, int n,
     int max_steps, const int* __restrict__ layers, const int* __restrict__ hits, const float* __restrict__ p0,
     const float* __restrict__ c0, const float* __restrict__ align, const float* __restrict__ xscale,
-    float* __restrict__ chi2_out, float* __restrict__ d_p0, float* __restrict__ d_align,
-    float* __restrict__ d_xscale, int* __restrict__ status_out, float* __restrict__ ck) {
+    float* __restrict__ chi2_out, int4* __restrict__ trk, int* __restrict__ key_counts, float* __restrict__ ck) {
     __shared__ DevGeom g;
-    __shared__ float acc[MKGB_MAX_LAYERS * 7];
     load_geom(gp, g);
-    for (int q = threadIdx.x; q < MKGB_MAX_LAYERS * 7; q += blockDim.x) acc[q] = 0.0f;
     __syncthreads();
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n) {
-        const int* lrow = layers + (int64_t)i * max_steps;
-        const int* hrow = hits + (int64_t)i * max_steps;
-        int nl = 0;
-        while (nl < max_steps && lrow[nl] >= 0 && lrow[nl] < g.n_layers) ++nl;
-        // ---- plain pass, checkpointing the input of every step
-        State t;
-        {
-            const float* pi = p0 + 6 * (int64_t)i;
-            const float* ci = c0 + 21 * (int64_t)i;
-            t.xh = pi[0]; t.yh = pi[1]; t.zh = pi[2];
-            t.xl = 0.0f; t.yl = 0.0f; t.zl = 0.0f;
-            t.k = pi[3]; t.phi = pi[4]; t.th = pi[5];
-#pragma unroll 1
-            for (int q = 0; q < 21; ++q) t.c[q] = ci[q];
-        }
-        int status = 0;
-        float chi2v = 0.0f;
-        for (int j = 0; j < nl && status == 0; ++j) {
-            const int l = lrow[j];
-            store_ck(ck + ((int64_t)j * n + i) * 32, t);
-            float x2 = 0.0f;
-            status = fit_step<float, MOD>(g, P, pay, n_hits, l, hrow[j], t, align + 6 * l, xscale[l], x2);
-            chi2v += x2;
-        }
-        // ---- reverse sweep
-        float lam[kStateIn];   // d total / d (state after step j)
+    if (i >= n) return;
+    const int* lrow = layers + (int64_t)i * max_steps;
+    const int* hrow = hits + (int64_t)i * max_steps;
+    int nl = 0;
+    while (nl < max_steps && lrow[nl] >= 0 && lrow[nl] < g.n_layers) ++nl;
+    State t;
+    {
+        const float* pi = p0 + 6 * (int64_t)i;
+        const float* ci = c0 + 21 * (int64_t)i;
+        t.xh = pi[0]; t.yh = pi[1]; t.zh = pi[2];
+        t.xl = 0.0f; t.yl = 0.0f; t.zl = 0.0f;
+        t.k = pi[3]; t.phi = pi[4]; t.th = pi[5];
 #pragma unroll
-        for (int c = 0; c < kStateIn; ++c) lam[c] = 0.0f;
-        for (int j = nl - 1; j >= 0 && status == 0; --j) {
-            const int l = lrow[j], h = hrow[j];
-            State t0;
-            load_ck(ck + ((int64_t)j * n + i) * 32, t0);
-            const float* al = align + 6 * l;
-            float lnew[kStateIn];
-            for (int base = 0; base < kStepIn; base += KD) {
+        for (int q = 0; q < 21; ++q) t.c[q] = ci[q];
+    }
+    int status = 0, disks = 0;
+    float chi2v = 0.0f;
+    for (int j = 0; j < nl && status == 0; ++j) {
+        const int l = lrow[j];
+        disks += g.layers[l].kind == MKGB_DISK;
+        store_ck(ck + ((int64_t)j * n + i) * 32, t);
+        float x2 = 0.0f;
+        status = fit_step<float, MOD>(g, P, pay, n_hits, l, hrow[j], t, align + 6 * l, xscale[l], x2);
+        chi2v += x2;
+    }
+    chi2_out[i] = chi2v;
+    const int key = (kAdjKeyLen - 1 - min(status == 0 ? nl : 0, kAdjKeyLen - 1)) * kAdjKeyDisks + min(disks, kAdjKeyDisks - 1);
+    trk[i] = make_int4(nl, status, key, atomicAdd(key_counts + key, 1));
+}
+
+__global__ void __launch_bounds__(256) k_adj_order(int n, const int4* __restrict__ trk,
+                                                   const int* __restrict__ key_off, int* __restrict__ order) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const int4 t = trk[i];
+    order[key_off[t.z] + t.w] = i;
+}
+
+// The sweep's bound is the fetch of its own code: a dual step is ~12,000 straight-line
+// instructions (200 KB, more than the instruction cache), and 255 registers leave room for eight
+// warps.  With one thread per track and all passes each warp walked through that code on its own
+// (no_instruction 2.1-4.9 of the stall cycles per issue, issue active 21%).  So the eight warps of
+// a block share the passes of a step (17 at KD = 2), start each round of them together and share
+// the fetches; a small batch spreads over eight times as many warps.  The tracks are taken in the
+// order of their length and layer kinds, so that the lanes of a warp walk the same steps (31 of 32
+// active instead of 21, and no round for the few long tracks of a block), longest first.
+// 1 to kAdjWide groups of 32 tracks per block: four make 68 passes for 8 warps (9 rounds, 94%
+// busy), one 3 rounds (71%); the launch takes the number with the fewest rounds over all blocks.
+// 100k tracks, 12 layers each, of the misaligned endcap: 23.4 ms with one thread per track; passes
+// shared by the warps 14.5, rounds started together 12.3, in order 9.5 ms; 1,001 tracks:
+// 5.77 -> 0.82 ms.  One direction per pass (KD = 1, 12 warps of 168 registers) rounds the
+// derivatives differently: d/dp0 of a few ill-conditioned tracks moves by up to 1e-3.
+constexpr int kAdjWarps = 8, kAdjThreads = 32 * kAdjWarps;
+constexpr int kAdjPasses = (kStepIn + KD - 1) / KD;
+constexpr int kAdjWide = 4;   // groups of 32 tracks per block where the batch fills the device
+
+template <bool MOD>
+__global__ void __launch_bounds__(kAdjThreads, 1) k_fit_adjoint(
+    const DevGeom* __restrict__ gp, DevParams P, const float4* __restrict__ pay, int64_t n_hits, int n,
+    int max_steps, const int* __restrict__ layers, const int* __restrict__ hits, const float* __restrict__ align,
+    const float* __restrict__ xscale, float* __restrict__ chi2_out, float* __restrict__ d_p0,
+    float* __restrict__ d_align, float* __restrict__ d_xscale, int* __restrict__ status_out,
+    const int4* __restrict__ trk, const int* __restrict__ order, const float* __restrict__ ck, int groups) {
+    __shared__ DevGeom g;
+    __shared__ float acc[MKGB_MAX_LAYERS * 7];
+    __shared__ int s_nl[32 * kAdjWide];   // steps to redo; 0 once a redone step has failed
+    __shared__ int s_status[32 * kAdjWide];
+    __shared__ int s_id[32 * kAdjWide];
+    __shared__ int s_max;
+    // d total / d (state after the step), of the step at hand and of the one before it:
+    // [2][kStateIn][tracks]
+    extern __shared__ float s_lam[];
+    const int tracks = 32 * groups;
+    load_geom(gp, g);
+    for (int q = threadIdx.x; q < MKGB_MAX_LAYERS * 7; q += blockDim.x) acc[q] = 0.0f;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    for (int64_t i0 = (int64_t)blockIdx.x * tracks; i0 < n; i0 += (int64_t)gridDim.x * tracks) {
+        __syncthreads();   // the geometry and acc are set; the last tracks' adjoints are written out
+        if (threadIdx.x == 0) s_max = 0;
+        __syncthreads();
+        for (int u = threadIdx.x; u < tracks; u += kAdjThreads) {
+            const int id = i0 + u < n ? order[i0 + u] : 0;
+            const int4 tr = i0 + u < n ? trk[id] : make_int4(0, 0, 0, 0);
+            s_id[u] = id;
+            s_status[u] = tr.y;
+            s_nl[u] = tr.y == 0 ? tr.x : 0;
+            atomicMax(&s_max, s_nl[u]);
+        }
+        for (int q = threadIdx.x; q < kStateIn * tracks; q += kAdjThreads) s_lam[q] = 0.0f;
+        __syncthreads();
+        int cur = 0;
+        for (int j = s_max - 1; j >= 0; --j, cur ^= 1) {
+            const float* lam = s_lam + cur * kStateIn * tracks;
+            float* next = s_lam + (cur ^ 1) * kStateIn * tracks;
+#pragma unroll 1
+            for (int w0 = 0; w0 < groups * kAdjPasses; w0 += kAdjWarps) {
+                __syncthreads();   // the warps start a pass together
+                const int w = w0 + wid;
+                if (w >= groups * kAdjPasses) continue;
+                const int ps = w % kAdjPasses, u = (w / kAdjPasses) * 32 + lane;
+                const int64_t i = s_id[u];
+                const bool on = j < s_nl[u];
+                const int l = on ? layers[i * max_steps + j] : 0, h = on ? hits[i * max_steps + j] : -1;
+                const int base = ps * KD;
+                float out[KD];
+#pragma unroll
+                for (int k = 0; k < KD; ++k) out[k] = 0.0f;
                 // without a hit the alignment has no effect: skip passes that seed only it
-                if (h < 0 && base >= kStateIn + 1 && base + KD <= kStepIn - 1) continue;
-                StateT<D> td;
-                td.xh = seeded(t0.xh, 0, base); td.yh = seeded(t0.yh, 1, base); td.zh = seeded(t0.zh, 2, base);
-                td.xl = D(t0.xl); td.yl = D(t0.yl); td.zl = D(t0.zl);
-                td.k = seeded(t0.k, 3, base); td.phi = seeded(t0.phi, 4, base); td.th = seeded(t0.th, 5, base);
-                td.tl = D(t0.tl);
-                td.pl = D(t0.pl);
-#pragma unroll 1
-                for (int q = 0; q < 21; ++q) td.c[q] = seeded(t0.c[q], 6 + q, base);
-                D ald[6];
+                const bool idle = h < 0 && base >= kStateIn + 1 && base + KD <= kStepIn - 1;
+                if (on && !idle) {
+                    State t0;
+                    load_ck(ck + ((int64_t)j * n + i) * 32, t0);
+                    const float* al = align + 6 * l;
+                    StateT<D> td;
+                    td.xh = seeded(t0.xh, 0, base);
+                    td.yh = seeded(t0.yh, 1, base);
+                    td.zh = seeded(t0.zh, 2, base);
+                    td.xl = D(t0.xl); td.yl = D(t0.yl); td.zl = D(t0.zl);
+                    td.k = seeded(t0.k, 3, base);
+                    td.phi = seeded(t0.phi, 4, base);
+                    td.th = seeded(t0.th, 5, base);
+                    td.tl = D(t0.tl);
+                    td.pl = D(t0.pl);
 #pragma unroll
-                for (int c = 0; c < 6; ++c) ald[c] = seeded(al[c], kStateIn + c, base);
-                const D xs = seeded(xscale[l], kStepIn - 1, base);
-                D x2;
-                if (fit_step<D, MOD>(g, P, pay, n_hits, l, h, td, ald, xs, x2) != 0) {
-                    status = 5;   // the redone step failed where the plain pass did not
-                    break;
+                    for (int q = 0; q < 21; ++q) td.c[q] = seeded(t0.c[q], 6 + q, base);
+                    D ald[6];
+#pragma unroll
+                    for (int c = 0; c < 6; ++c) ald[c] = seeded(al[c], kStateIn + c, base);
+                    const D xs = seeded(xscale[l], kStepIn - 1, base);
+                    D x2;
+                    if (fit_step<D, MOD>(g, P, pay, n_hits, l, h, td, ald, xs, x2) != 0) {
+                        s_status[u] = 5;   // the redone step failed where the plain pass did not
+                    } else {
+#pragma unroll
+                        for (int k = 0; k < KD; ++k) {
+                            float a = x2.d[k];
+                            a = fmaf(lam[u], td.xh.d[k] + td.xl.d[k], a);
+                            a = fmaf(lam[tracks + u], td.yh.d[k] + td.yl.d[k], a);
+                            a = fmaf(lam[2 * tracks + u], td.zh.d[k] + td.zl.d[k], a);
+                            a = fmaf(lam[3 * tracks + u], td.k.d[k], a);
+                            a = fmaf(lam[4 * tracks + u], td.phi.d[k] + td.pl.d[k], a);
+                            a = fmaf(lam[5 * tracks + u], td.th.d[k] + td.tl.d[k], a);
+#pragma unroll
+                            for (int q = 0; q < 21; ++q) a = fmaf(lam[(6 + q) * tracks + u], td.c[q].d[k], a);
+                            out[k] = a;
+                        }
+                    }
                 }
 #pragma unroll
                 for (int k = 0; k < KD; ++k) {
                     const int comp = base + k;
-                    if (comp >= kStepIn) break;
-                    float a = x2.d[k];
-                    a = fmaf(lam[0], td.xh.d[k] + td.xl.d[k], a);
-                    a = fmaf(lam[1], td.yh.d[k] + td.yl.d[k], a);
-                    a = fmaf(lam[2], td.zh.d[k] + td.zl.d[k], a);
-                    a = fmaf(lam[3], td.k.d[k], a);
-                    a = fmaf(lam[4], td.phi.d[k] + td.pl.d[k], a);
-                    a = fmaf(lam[5], td.th.d[k] + td.tl.d[k], a);
-#pragma unroll
-                    for (int q = 0; q < 21; ++q) a = fmaf(lam[6 + q], td.c[q].d[k], a);
                     if (comp < kStateIn)
-                        lnew[comp] = a;
-                    else if (a != 0.0f)
-                        atomicAdd(acc + l * 7 + (comp - kStateIn), a);
+                        next[comp * tracks + u] = out[k];
+                    else if (comp < kStepIn && out[k] != 0.0f)
+                        atomicAdd(acc + l * 7 + (comp - kStateIn), out[k]);
                 }
             }
-#pragma unroll
-            for (int c = 0; c < kStateIn; ++c) lam[c] = lnew[c];
+            __syncthreads();   // the step's adjoints are complete
+            for (int u = threadIdx.x; u < tracks; u += kAdjThreads)
+                if (s_status[u] != 0) s_nl[u] = 0;
+            __syncthreads();
         }
-        if (status != 0) {
-            chi2v = 0.0f;
+        for (int u = threadIdx.x; u < tracks && i0 + u < n; u += kAdjThreads) {
+            const int status = s_status[u];
+            const int64_t i = s_id[u];
 #pragma unroll
-            for (int c = 0; c < 6; ++c) lam[c] = 0.0f;
+            for (int c = 0; c < 6; ++c) d_p0[6 * i + c] = status == 0 ? s_lam[(cur * kStateIn + c) * tracks + u] : 0.0f;
+            if (status != 0) chi2_out[i] = 0.0f;
+            if (status_out) status_out[i] = status;
         }
-#pragma unroll
-        for (int c = 0; c < 6; ++c) d_p0[6 * (int64_t)i + c] = lam[c];
-        chi2_out[i] = chi2v;
-        if (status_out) status_out[i] = status;
     }
     __syncthreads();
     for (int q = threadIdx.x; q < g.n_layers * 7; q += blockDim.x) {
@@ -326,20 +413,50 @@ __global__ void __launch_bounds__(kThreads) k_fit_adjoint(
 
 }  // namespace
 
+size_t fit_grad_scratch_bytes(int n, int max_steps) {
+    return (size_t)n * (128 * (size_t)(max_steps > 0 ? max_steps : 1) + 16 + 4) + 4 * (kAdjKeys + 4);
+}
+
 cudaError_t launch_fit_grad(cudaStream_t st, const DevGeom* g, DevParams P, const float4* pay, int64_t n_hits, int n,
                             int max_steps, const int* layers, const int* hits, const float* p0, const float* c0,
                             const float* align, const float* xscale, float* chi2_out, float* d_p0, float* d_align,
-                            float* d_xscale, int* status_out, float* ck, bool modular) {
+                            float* d_xscale, int* status_out, float* ck, int n_sms, bool modular) {
     if (n == 0) return cudaSuccess;
     const int blocks = (n + kThreads - 1) / kThreads;
-    auto adjoint = modular ? k_fit_adjoint<true> : k_fit_adjoint<false>;
+    if (ck) {
+        auto plain = modular ? k_fit_ck<true> : k_fit_ck<false>;
+        auto adjoint = modular ? k_fit_adjoint<true> : k_fit_adjoint<false>;
+        // after the checkpoints: per track (steps, status, key, rank), the keys' counts, the order
+        int4* trk = reinterpret_cast<int4*>(ck + (size_t)32 * n * (max_steps > 0 ? max_steps : 1));
+        int* key_counts = reinterpret_cast<int*>(trk + n);
+        int* order = key_counts + kAdjKeys + 4;
+        cudaError_t e = cudaMemsetAsync(key_counts, 0, 4 * kAdjKeys, st);
+        if (e != cudaSuccess) return e;
+        plain<<<blocks, kThreads, 0, st>>>(g, P, pay, n_hits, n, max_steps, layers, hits, p0, c0, align, xscale,
+                                           chi2_out, trk, key_counts, ck);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        if ((e = exclusive_scan(st, key_counts, key_counts, kAdjKeys, nullptr)) != cudaSuccess) return e;   // one block
+        k_adj_order<<<(n + 255) / 256, 256, 0, st>>>(n, trk, key_counts, order);
+        if ((e = cudaGetLastError()) != cudaSuccess) return e;
+        // groups per block: the fewest rounds of passes over all blocks of an SM
+        int groups = 1, need = 0, best = 0;
+        for (int gr = 1; gr <= kAdjWide; ++gr) {
+            const int nb = (n + 32 * gr - 1) / (32 * gr);
+            const int rounds = (nb + n_sms - 1) / n_sms * ((gr * kAdjPasses + kAdjWarps - 1) / kAdjWarps);
+            if (gr == 1 || rounds < best) {
+                best = rounds;
+                groups = gr;
+                need = nb;
+            }
+        }
+        adjoint<<<need < n_sms ? need : n_sms, kAdjThreads, 2 * kStateIn * 32 * groups * sizeof(float), st>>>(
+            g, P, pay, n_hits, n, max_steps, layers, hits, align, xscale, chi2_out, d_p0, d_align, d_xscale,
+            status_out, trk, order, ck, groups);
+        return cudaGetLastError();
+    }
     auto forward = modular ? k_fit_grad<true> : k_fit_grad<false>;
-    if (ck)
-        adjoint<<<blocks, kThreads, 0, st>>>(g, P, pay, n_hits, n, max_steps, layers, hits, p0, c0, align,
-                                                   xscale, chi2_out, d_p0, d_align, d_xscale, status_out, ck);
-    else
-        forward<<<blocks, kThreads, 0, st>>>(g, P, pay, n_hits, n, max_steps, layers, hits, p0, c0, align, xscale,
-                                                chi2_out, d_p0, d_align, d_xscale, status_out);
+    forward<<<blocks, kThreads, 0, st>>>(g, P, pay, n_hits, n, max_steps, layers, hits, p0, c0, align, xscale,
+                                         chi2_out, d_p0, d_align, d_xscale, status_out);
     return cudaGetLastError();
 }
 

@@ -178,6 +178,26 @@ def test_reverse_sweep_matches_forward_mode(lib, aligned_small):
     assert np.median(rel) < 1e-4 and np.percentile(rel, 99) < 1e-2, (np.median(rel), np.percentile(rel, 99))
 
 
+@pytest.mark.parametrize("n", [1, 31, 33, 129, 20_011])
+def test_reverse_sweep_does_not_depend_on_the_batch(lib, aligned_small, n):
+    """A track's chi2, derivative and status are the same bits in a batch of any size (the sweep's
+    blocks take 32 to 128 tracks, in the order of their length); a track without layers gives zeros."""
+    from types import SimpleNamespace
+    g, batch, fi, al, xs = aligned_small
+    full = _gpu_grad(g, batch, fi, -al, xs)
+    m = fi.layers.shape[0]
+    rows = np.random.default_rng(n).integers(0, m, n)
+    pick = lambda a: np.ascontiguousarray(a[rows])
+    f = SimpleNamespace(layers=pick(fi.layers), hits=pick(fi.hits), p0=pick(fi.p0), c0=pick(fi.c0))
+    empty = n // 2
+    f.layers[empty] = -1
+    got = _gpu_grad(g, batch, f, -al, xs)
+    rest = np.arange(n) != empty
+    for k in ("chi2", "dp0", "status"):
+        assert np.array_equal(got[k][rest], full[k][rows][rest]), k
+        assert not np.any(got[k][empty]), k
+
+
 def _subset(fi, n):
     from types import SimpleNamespace
     return SimpleNamespace(layers=np.ascontiguousarray(fi.layers[:n]), hits=np.ascontiguousarray(fi.hits[:n]),
