@@ -291,11 +291,10 @@ int mkgb_run_modular(mkgb_ctx* ctx, int n_events, const int64_t* seg_off, const 
 
 /* Launch configuration of the search rounds (mkgb_build, mkgb_run).  The paper has no
  * counterpart: this is a library service that changes neither results nor arithmetic.
- * find_shape picks how a round of the search runs: 0, 1, 2 as two kernels per plan step (one
- * thread per candidate for propagation, window and chi2; eight lanes per seed for the merge and
- * the update) with blocks of 128, 64 or 256 threads for the first kernel and select_shape (0, 1,
- * 2: 128, 64, 256 threads) for the second; 3, 4, 5 as one fused kernel per plan step (blocks of
- * 128 threads with 4 or 3 resident per SM, or 256 threads with 2; select_shape is ignored).
+ * A round of the search runs as three kernels (a candidate's update and propagation; its window
+ * and chi2; the merge per seed).  find_shape 0..5 picks the blocks of the first: 128, 128, 256, 64,
+ * 64 or 128 threads with 5, 4, 2, 8, 10 or 3 of them resident per SM; select_shape 0..2 those of
+ * the second: 128, 64 or 128 threads with 6, 12 or 8.  (1, 0) is the default.
  * Each kernel launches as many blocks as stay resident on the device.  use_graph = 1 (the
  * default) records the launches of one search as a CUDA graph on the first call and replays it
  * while the arguments, shapes and stream stay the same (a change re-records); the graph is used
@@ -306,8 +305,8 @@ int mkgb_run_modular(mkgb_ctx* ctx, int n_events, const int64_t* seg_off, const 
 int mkgb_set_launch(mkgb_ctx* ctx, int find_shape, int select_shape, int use_graph);
 
 /* Autotuner of the search launch shapes (library service, no counterpart in the paper): runs
- * the search over the seeds loaded now (mkgb_seed) once per launch configuration (the 3 x 3
- * two-kernel pairs and the 3 fused shapes of mkgb_set_launch), each warmed once and then timed
+ * the search over the seeds loaded now (mkgb_seed) once per launch configuration (the 6 x 3
+ * shapes of mkgb_set_launch), each warmed once and then timed
  * reps times with CUDA events on the context's stream, keeps the fastest as the context's
  * shapes (mkgb_set_launch) and writes it to find_shape / select_shape (may be NULL) and its mean
  * time per search to ms_out (may be NULL).  The outputs of these searches go to the library's

@@ -23,6 +23,7 @@ ARCH = ["-gencode", "arch=compute_103a,code=sm_103a"]
 # 2 ulp instead of 0.5: well inside the error budget of the FP32 step, ~5% faster search);
 # FP64 arithmetic is not affected by these flags.
 FILE_FLAGS = {"k_build.cu": ["-prec-div=false", "-prec-sqrt=false"],
+              "k_build_mod.cu": ["-prec-div=false", "-prec-sqrt=false"],
               "k_fit.cu": ["-prec-div=false", "-prec-sqrt=false"]}
 FLAGS = ["-O3", "-lineinfo", "-std=c++17", "-Xcompiler", "-fPIC", "-I", INCLUDE, "-I", CSRC,
          "--expt-relaxed-constexpr"]

@@ -93,7 +93,7 @@ struct mkgb_ctx {
     bool mod_hits = false;
     DevBuf stage[S_COUNT];
     // launch shapes of the search rounds and the graph cache replaying them
-    int find_shape = 1, select_shape = 0;   // two kernels per round: find 64 x 8, select 128 x 5
+    int find_shape = 1, select_shape = 0;   // k_move 128 x 4, k_find 128 x 6
     bool use_graph = true;
     BuildGraph* graph = nullptr;
 };
@@ -211,9 +211,8 @@ int enqueue_build(mkgb_ctx* ctx, const BuildOutDev& d, int find_shape, int selec
     const int prec = ctx->params.precision;
     if (prec == MKGB_FP64 && !ctx->seeds_fp64)
         return fail(ctx, MKGB_ESTATE, "FP64 search needs seeds made under the FP64 precision");
-    const bool ovl = ctx->mod_hits;   // overlap hits need their own trail
-    CK(ensure(ctx->build_work, build_work_bytes(ctx->n_seeds, ctx->max_plan_len, prec, ovl)));
-    const BuildWork w = carve_build_work(ctx->build_work.p, ctx->n_seeds, ctx->max_plan_len, prec, ovl);
+    CK(ensure(ctx->build_work, build_work_bytes(ctx->n_seeds, ctx->max_plan_len, prec, ctx->mod_hits)));
+    const BuildWork w = carve_build_work(ctx->build_work.p, ctx->n_seeds, ctx->max_plan_len, prec, ctx->mod_hits);
     CK(cudaMemsetAsync(ctx->counters_build.p, 0, 8 * kNumCounters, st));
     if (ctx->use_graph && !ctx->graph) ctx->graph = build_graph_create();
     CK(launch_build(st, (const DevGeom*)ctx->geom_d.p, ctx->max_plan_len, ctx->params, hit_store(ctx), S, d, w,
@@ -738,7 +737,7 @@ int mkgb_build_backward(mkgb_ctx* ctx, int n, const int32_t* track_event, const 
     const BuildWork w = carve_build_work(ctx->build_work.p, n, ctx->max_plan_len, MKGB_FP32, ctx->mod_hits);
     CK(cudaMemsetAsync(ctx->counters_build.p, 0, 8 * kNumCounters, st));
     CK(launch_build(st, (const DevGeom*)ctx->geom_bwd_d.p, ctx->max_plan_len, ctx->params, hit_store(ctx), S, d, w,
-                    (unsigned long long*)ctx->counters_build.p, ctx->n_sms, ctx->find_shape >= 3 ? 3 : 0, 0, nullptr, true));
+                    (unsigned long long*)ctx->counters_build.p, ctx->n_sms, 1, 0, nullptr, true));
     CK(copy_back(ctx, out->params, d.params, 24 * N, on_device));
     CK(copy_back(ctx, out->cov, d.cov, 84 * N, on_device));
     CK(copy_back(ctx, out->chi2, d.chi2, 4 * N, on_device));
@@ -1265,7 +1264,7 @@ int mkgb_autotune(mkgb_ctx* ctx, int reps, int* find_shape, int* select_shape, f
     int best_f = ctx->find_shape, best_s = ctx->select_shape, rc = MKGB_OK;
     float best = -1.0f;
     for (int f = 0; f < 6 && rc == MKGB_OK; ++f)
-        for (int s = 0; s < (f < 3 ? 3 : 1) && rc == MKGB_OK; ++s) {   // fused shapes have no select kernel
+        for (int s = 0; s < 3 && rc == MKGB_OK; ++s) {
             rc = enqueue_build(ctx, d, f, s);   // warm-up (and the graph's recording)
             if (rc == MKGB_OK) cudaEventRecord(e0, st);
             for (int r = 0; r < reps && rc == MKGB_OK; ++r) rc = enqueue_build(ctx, d, f, s);

@@ -9,7 +9,7 @@
 namespace mk {
 
 // Child kinds of a candidate at one layer (a10).
-enum : int { K_NONE = 0, K_HIT = 1, K_MISS = 2, K_SKIP = 3, K_STOP = 4, K_CARRY = 5 };
+enum : int { K_NONE = 0, K_HIT = 1, K_MISS = 2, K_SKIP = 3, K_STOP = 4, K_CARRY = 5, K_SEED = 6 };
 
 constexpr int kSeedStateStride = 32;   // xh,yh,zh,xl,yl,zl,k,phi,th,c[21],pad,pad
 constexpr int kSeedEtaCells = 32;      // coarse eta-phi cells for the seed order (a3)
@@ -47,27 +47,30 @@ struct BuildOutDev {
     int* ovl = nullptr;   // n x max_plan overlap hit ids (-1 none), nullptr: not wanted
 };
 
-// Work buffers of the search (k_build.cu): per seed 8 candidate slots, double-buffered.
+// Work buffers of the search (k_build.cu): per seed 8 candidate slots, in tiles of 32 seeds (slot_at,
+// word_at there).
 struct BuildWork {
-    unsigned char* st[2];   // slot states, 32 words (FP32 or FP64 per the precision)
-    int4* meta[2];    // slot (score, chi2 sum, nfound | nholes << 8 | stopped << 16, alive)
-    unsigned char* pr;      // slot predictions at the round's layer, 28 words
-    // slot children: (n hits, non-hit kind, non-hit score, b2) + 4 x (chi2, hit, chi2, hit); b2: with
-    // module hits, the best accepted hit on another module than the first entry's (-1 none)
+    // slot records, 32 words (FP32 or FP64 per the precision): a candidate's prediction at its round's
+    // layer, or its state where it did not cross it; written in turn by even and odd rounds
+    unsigned char* rec[2];
+    unsigned char* stop;   // records put aside: the predictions at which a seed's stopped candidates stopped
+    // slot (score, chi2 sum, nfound | nholes << 8 | stopped << 16 | stopped on a disk << 17 | place of its
+    // stop record << 18, alive)
+    int4* meta[2];
+    int4* child;      // slot's child descriptor: (parent slot | kind << 4 | disk << 8, hit or seed, score, nholes)
+    // slot children: (n hits | disk, non-hit kind, non-hit score, -) + (chi2, hit, chi2, hit)
     int4* ls;
+    int4* ls_more;    // 3 x (chi2, hit, chi2, hit): the third to eighth hit
     int* live[2];     // work list of live candidate slots per round
     int* seeds[2];    // work list of seeds with a live candidate per round
     int4* sinfo;      // per ordered seed: (plan position of its first step, first step, steps, event)
-    int* fin;         // per ordered seed: buffer holding its final slots | (rounds searched << 1), -1 none
-    int* trail;       // per ordered seed: longest plan x 8 ints ((code + 4) << 3 | parent slot)
-    int* otrail;      // the same layout: overlap hit id of the step (-1 none); nullptr without modules
-    int* rescue;      // kept children of the round whose update is redone in FP64
-    int* counts;      // [live0, live1, seeds0, seeds1, rescue]
-    // fused rounds: [tau] length of round tau's live list, [kRescueCountBase + tau] its FP64 redo list
-    int* rcounts;
+    int* fin;         // per ordered seed: rounds searched, -1 none
+    int* trail;       // per round and slot ((code + 4) << 3 | parent slot); a hit's code is its binned index
+    int* redo;        // children of the round whose update is redone in FP64
+    int* found;       // candidates of the round that crossed their layer
+    int* counts;      // [live0, live1, seeds0, seeds1, redo, found]
+    void* mod;        // not nullptr: module hits are loaded, the search is k_build_mod.cu's and this its work
 };
-constexpr int kRescueCountBase = MKGB_MAX_PLAN + 2;
-constexpr int kRoundCountInts = 2 * kRescueCountBase;
 
 // counters (64-bit): [0] steps, [1] chi2 evaluations, [2] updates, [3] hits tested, [4] Newton iterations
 constexpr int kNumCounters = 5;
@@ -116,9 +119,16 @@ cudaError_t launch_seed_keys(cudaStream_t st, int n, const float* state, const i
                              int* key_counts);
 
 // ---- k_build.cu
-// with_ovl: room for the overlap hits of modular layers (the otrail array)
-size_t build_work_bytes(int n_seeds, int max_plan_len, int precision, bool with_ovl = false);
-BuildWork carve_build_work(void* base, int n_seeds, int max_plan_len, int precision, bool with_ovl = false);
+// modular: module hits are loaded
+size_t build_work_bytes(int n_seeds, int max_plan_len, int precision, bool modular = false);
+BuildWork carve_build_work(void* base, int n_seeds, int max_plan_len, int precision, bool modular = false);
+// ---- k_build_mod.cu: the rounds with module hits; work of mod_work_bytes
+size_t mod_work_bytes(int n_seeds, int max_plan_len, int precision);
+void prime_mod_shapes(int precision, int n_sms);
+cudaError_t launch_mod_rounds(cudaStream_t st, const DevGeom* g, int max_plan_len, DevParams P, HitStore H, SeedStore S,
+                              BuildOutDev out, void* work, unsigned long long* counters, int n_sms, int find_shape,
+                              int select_shape, bool backward);
+// ---- k_build.cu
 struct BuildGraph;
 BuildGraph* build_graph_create();
 void build_graph_destroy(BuildGraph* gph);

@@ -1,28 +1,35 @@
-// Combinatorial forward search (Sec. 2.2) as layer-synchronous rounds of two kernels.
+// Combinatorial forward search (Sec. 2.2) as layer-synchronous rounds of three kernels.
 //
 // All seeds of all events advance together, one step of their layer plan per round (the
 // paper's search processes every candidate of a layer before the next, Sec. 3.1).  A seed owns
 // 8 candidate slots; per round:
-//   k_find    one thread per live candidate, taken from a compacted work list: propagation with
-//             Jacobian, transport and material (a4-a7), the eta-phi window (a8) and the chi2 of
-//             each hit inside it (a9).  Writes the predicted state (surface frame) and the
-//             candidate's children: its best hits (chi2 asc, hit id asc) and its non-hit child;
-//   k_select  eight lanes per seed (lane = parent slot): merges the children of the seed's
-//             candidates into the N best with 64-bit (score, parent slot) keys reduced by warp
-//             shuffles (a10); lane r takes the r-th child, applies the Joseph update with its hit
-//             from the parent's prediction (a11), writes slot r of the next round's buffers and
-//             (parent slot, hit) to the trail, and appends the child to the next work lists.
-// k_start fills round 0 from the seed states; k_finish picks each seed's best candidate and walks
-// the trail back for its hit list (a13).
+//   k_move    one thread per live child, taken from a compacted work list: its state from its
+//             parent's prediction and its hit (the Joseph update, a11), then the propagation to the
+//             round's layer with Jacobian, transport and material (a4-a7);
+//   k_find    one thread per child that crossed the layer: the eta-phi window (a8) and the chi2 of
+//             each hit inside it (a9).  Writes the candidate's own children: its best hits (chi2
+//             asc, hit id asc) and its non-hit child;
+//   k_merge   eight lanes per seed: the N best children over the seed's candidates (a10), their
+//             descriptors (parent slot, hit), (parent slot, hit) for the trail, the next work lists.
+// k_start makes each seed the first child of its slot 0; k_finish gives each seed's best child its
+// state and walks the trail back for its hit list (a13).
 //
-// Slot records are array-of-structures in HBM: a state is 32 floats (xh, yh, zh, xl, yl, zl, k,
-// phi, theta, 21 covariance terms, theta's and phi's low parts), a prediction 28 floats, a child
-// list 20 ints, the slot's (score, chi2 sum, counts, alive) one int4.  With module hits loaded
-// (Sec. 3.1), the child list also names the best accepted hit on another module than its first
-// entry's, and an overlap trail beside the hit trail keeps each step's overlap hit (Sec. 2.2).  Work lists are filled with warp-aggregated
-// atomics, so the threads of a warp read neighbouring slots.  No kernel waits on another block;
-// every loop is bounded by a list length, a window's bin range or the Newton iteration limit.
+// Why three kernels: k_move computes (128 registers a thread, 16 warps per SM), k_find waits for
+// chains of small loads and k_merge for short lists, and both need warps.  A child's state exists in
+// registers only: its update and its propagation follow each other in k_move, one thread per child,
+// and only predictions go through HBM.  The former round (propagation and window in one kernel, then
+// merge and update by eight lanes per seed, 18.5 of 32 lanes active, states and predictions both
+// written, records one after another) took 21.6 ms for 64 Phase-2-like events (1.28M seeds, 58M
+// crossed steps) and 0.90 ms for one; one kernel for update, propagation and window 17.2 ms (its 128
+// registers also held the window's chains of loads to 16 warps); these three 15.9 and 0.66 ms:
+// k_move 7.4 ms, k_find 2.9, k_merge 4.8 of the 64 events.  k_move is bound by issue and latency
+// together (47% issue active, 28% of DRAM), k_find and k_merge by their dependent loads.
+//
+// No kernel waits on another block; every loop is bounded by a list length, a window's bin range or
+// the Newton iteration limit.  The kernels of a search are chained by programmatic dependent
+// launches: a kernel's blocks start and load the geometry while the one before it ends.
 #include "internal.h"
+#include "launch.cuh"
 
 #include <cstring>
 
@@ -33,19 +40,11 @@ namespace {
 constexpr int kGroup = 8;   // slots (lanes) per seed, >= MKGB_MAX_CANDS
 constexpr int kThreads = 128;
 constexpr float kBig = 3.0e38f;
+constexpr int kQueue = 8;
+constexpr int kDiskBit = 16;   // in a child list's header beside the number of hits: its layer is a disk
 constexpr unsigned kFull = 0xffffffffu;
 
-__device__ __forceinline__ unsigned long long order_key(float score, int slot) {
-    unsigned u = __float_as_uint(score);
-    u = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
-    return ((unsigned long long)u << 32) | (unsigned)(kGroup - 1 - slot);
-}
-
-__device__ __forceinline__ float shfl_f(float v, int src) { return __shfl_sync(kFull, v, src); }
-__device__ __forceinline__ int shfl_i(int v, int src) { return __shfl_sync(kFull, v, src); }
-
-// ---- slot records: a state is 32 words (xh, yh, zh, xl, yl, zl, k, phi, theta, 21 covariance
-// terms, theta's and phi's low parts), a prediction 28 words; words are F, moved as 16-byte vectors
+// ---- slot records: words of F, moved as 16-byte vectors
 
 __device__ __forceinline__ void unpack16(const float4& v, float* f) { f[0] = v.x; f[1] = v.y; f[2] = v.z; f[3] = v.w; }
 __device__ __forceinline__ void unpack16(const double2& v, double* f) { f[0] = v.x; f[1] = v.y; }
@@ -55,62 +54,47 @@ template <class F> struct Vec16;
 template <> struct Vec16<float> { using T = float4; };
 template <> struct Vec16<double> { using T = double2; };
 
-template <class F, int N> __device__ __forceinline__ void load_words(const unsigned char* __restrict__ p, F* f) {
-    using V = typename Vec16<F>::T;
-    constexpr int per = 16 / sizeof(F);
-    const V* v = reinterpret_cast<const V*>(p);
-#pragma unroll
-    for (int i = 0; i < N / per; ++i) unpack16(v[i], f + per * i);
+// Slots are laid out in tiles of 32 seeds: the 16-byte words of an array run over the seeds of a tile,
+// then over the eight slots, then over the words of a record.  A warp of k_move or k_merge, whose slots
+// come from a few neighbouring seeds, then touches about eight 128-byte lines per 16-byte load; with
+// one record after another each lane touched a line of its own, and the L1 handles one line per cycle
+// (~700 lines per warp of the update and propagation: 570 us a round of 640k seeds, 520 us in tiles).
+constexpr int kTile = 32;
+__host__ __device__ constexpr int tile_slots(int n_seeds) { return (n_seeds + kTile - 1) / kTile * (kTile * kGroup); }
+// Place of slot sl = seed * kGroup + slot in an array of one 16-byte word (or one int) per slot.
+__device__ __forceinline__ int slot_at(int sl) {
+    return (sl & ~(kTile * kGroup - 1)) | (sl & (kGroup - 1)) * kTile | ((sl / kGroup) & (kTile - 1));
+}
+// Place of word j of slot sl in an array of N words per slot.
+template <int N> __device__ __forceinline__ int64_t word_at(int sl, int j) {
+    return ((int64_t)(sl / (kTile * kGroup)) * N + j) * (kTile * kGroup) + (sl & (kGroup - 1)) * kTile +
+           ((sl / kGroup) & (kTile - 1));
 }
 
-template <class F, int N> __device__ __forceinline__ void store_words(unsigned char* __restrict__ p, const F* f) {
-    using V = typename Vec16<F>::T;
-    constexpr int per = 16 / sizeof(F);
-    V* v = reinterpret_cast<V*>(p);
-#pragma unroll
-    for (int i = 0; i < N / per; ++i) v[i] = pack16(f + per * i);
-}
-
-// Asynchronous 16-byte copy global -> shared (cached in L2 only), its commit and wait.
-__device__ __forceinline__ void cp_async16(void* smem, const void* gmem) {
-    const unsigned s = (unsigned)__cvta_generic_to_shared(smem);
-    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(s), "l"(gmem) : "memory");
-}
-__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
-
-// Words of a slot's state record (hi/lo positions, k, phi, theta, 21 covariance words, theta's
-// and phi's low parts) and of its prediction record (the same with 15 surface-frame covariance
-// words, padded to 16-byte words); layout_build_work sizes its arrays with them.
+// Words of a slot's record: a state (hi/lo positions, k, phi, theta, 21 covariance words, theta's and
+// phi's low parts) or a prediction (the same with 15 surface-frame covariance words).
 constexpr int kStateWords = 32, kPredWords = 28;
-static_assert(kStateWords == kSeedStateStride, "seed records are copied into state records");
+static_assert(kStateWords == kSeedStateStride, "seed records are read as state records");
+template <class F> constexpr int rec_vecs() { return (int)(kStateWords * sizeof(F) / 16); }
 template <class F> constexpr size_t state_bytes() { return kStateWords * sizeof(F); }
-template <class F> constexpr size_t pred_bytes() { return kPredWords * sizeof(F); }
 
-template <class F> __device__ __forceinline__ void load_state_rec(const unsigned char* r, StateT<F>& t) {
-    F f[kStateWords];
-    load_words<F, kStateWords>(r, f);
-    t.xh = f[0]; t.yh = f[1]; t.zh = f[2]; t.xl = f[3]; t.yl = f[4]; t.zl = f[5];
-    t.k = f[6]; t.phi = f[7]; t.th = f[8];
+template <class F, int W> __device__ __forceinline__ void load_rec(const unsigned char* __restrict__ base, int sl, F* f) {
+    using V = typename Vec16<F>::T;
+    constexpr int per = 16 / sizeof(F);
+    const V* v = reinterpret_cast<const V*>(base) + word_at<rec_vecs<F>()>(sl, 0);
 #pragma unroll
-    for (int i = 0; i < 21; ++i) t.c[i] = f[9 + i];
-    t.tl = f[30];
-    t.pl = f[31];
+    for (int j = 0; j < W / per; ++j) unpack16(v[j * (kTile * kGroup)], f + per * j);
 }
 
-template <class F> __device__ __forceinline__ void store_state_rec(unsigned char* r, const StateT<F>& t) {
-    F f[kStateWords];
-    f[0] = t.xh; f[1] = t.yh; f[2] = t.zh; f[3] = t.xl; f[4] = t.yl; f[5] = t.zl;
-    f[6] = t.k; f[7] = t.phi; f[8] = t.th;
+template <class F, int W> __device__ __forceinline__ void store_rec(unsigned char* __restrict__ base, int sl, const F* f) {
+    using V = typename Vec16<F>::T;
+    constexpr int per = 16 / sizeof(F);
+    V* v = reinterpret_cast<V*>(base) + word_at<rec_vecs<F>()>(sl, 0);
 #pragma unroll
-    for (int i = 0; i < 21; ++i) f[9 + i] = t.c[i];
-    f[30] = t.tl; f[31] = t.pl;
-    store_words<F, kStateWords>(r, f);
+    for (int j = 0; j < W / per; ++j) v[j * (kTile * kGroup)] = pack16(f + per * j);
 }
 
-template <class F> __device__ __forceinline__ void load_pred_rec(const unsigned char* r, PredT<F>& q) {
-    F f[kPredWords];
-    load_words<F, kPredWords>(r, f);
+template <class F> __device__ __forceinline__ void unpack_pred(const F* f, PredT<F>& q) {
     q.xh = f[0]; q.yh = f[1]; q.zh = f[2]; q.xl = f[3]; q.yl = f[4]; q.zl = f[5];
     q.k = f[6]; q.phi = f[7]; q.th = f[8];
 #pragma unroll
@@ -119,21 +103,57 @@ template <class F> __device__ __forceinline__ void load_pred_rec(const unsigned 
     q.pl = f[25];
 }
 
-template <class F> __device__ __forceinline__ void store_pred_rec(unsigned char* r, const PredT<F>& q) {
-    F f[kPredWords];
+template <class F> __device__ __forceinline__ void store_state_rec(unsigned char* base, int sl, const StateT<F>& t) {
+    F f[kStateWords];
+    f[0] = t.xh; f[1] = t.yh; f[2] = t.zh; f[3] = t.xl; f[4] = t.yl; f[5] = t.zl;
+    f[6] = t.k; f[7] = t.phi; f[8] = t.th;
+#pragma unroll
+    for (int i = 0; i < 21; ++i) f[9 + i] = t.c[i];
+    f[30] = t.tl; f[31] = t.pl;
+    store_rec<F, kStateWords>(base, sl, f);
+}
+
+// A prediction's record also holds the direction at the crossing (sin phi, cos phi, sin theta, cos
+// theta, as propagate_core returns it), for k_find.
+template <class F>
+__device__ __forceinline__ void store_pred_rec(unsigned char* base, int sl, const PredT<F>& q, const F dir[4]) {
+    F f[kStateWords];
     f[0] = q.xh; f[1] = q.yh; f[2] = q.zh; f[3] = q.xl; f[4] = q.yl; f[5] = q.zl;
     f[6] = q.k; f[7] = q.phi; f[8] = q.th;
 #pragma unroll
     for (int i = 0; i < 15; ++i) f[9 + i] = q.c[i];
-    f[24] = q.tl; f[25] = q.pl; f[26] = F(0); f[27] = F(0);
-    store_words<F, kPredWords>(r, f);
+    f[24] = q.tl; f[25] = q.pl;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) f[26 + i] = dir[i];
+    f[30] = F(0); f[31] = F(0);
+    store_rec<F, kStateWords>(base, sl, f);
 }
 
-template <class F> __device__ __forceinline__ void copy_state_rec(const unsigned char* src, unsigned char* dst) {
-    const float4* s4 = reinterpret_cast<const float4*>(src);
-    float4* d4 = reinterpret_cast<float4*>(dst);
+// The words of a prediction that the window and the chi2 take: positions, the
+// position covariance, the direction.
+template <class F>
+__device__ __forceinline__ void load_pred_rec(const unsigned char* __restrict__ base, int sl, PredT<F>& q, F dir[4]) {
+    using V = typename Vec16<F>::T;
+    constexpr int per = 16 / sizeof(F);
+    const V* v = reinterpret_cast<const V*>(base) + word_at<rec_vecs<F>()>(sl, 0);
+    F f[kStateWords];
 #pragma unroll
-    for (int q = 0; q < (int)(state_bytes<F>() / 16); ++q) d4[q] = s4[q];
+    for (int j = 0; j < kStateWords / per; ++j)
+        if (j * per < 12 || j * per >= 24) unpack16(v[j * (kTile * kGroup)], f + per * j);
+        else
+#pragma unroll
+            for (int i = 0; i < per; ++i) f[per * j + i] = F(0);
+    unpack_pred(f, q);
+#pragma unroll
+    for (int i = 0; i < 4; ++i) dir[i] = f[26 + i];
+}
+
+// The record of a seed (one after another, in the seeds' own order).
+template <class F> __device__ __forceinline__ void load_seed_rec(const F* __restrict__ r, F* f) {
+    using V = typename Vec16<F>::T;
+    constexpr int per = 16 / sizeof(F);
+#pragma unroll
+    for (int j = 0; j < kStateWords / per; ++j) unpack16(reinterpret_cast<const V*>(r)[j], f + per * j);
 }
 
 // slot meta: (score, chi2 sum, nfound | nholes << 8 | stopped << 16, alive)
@@ -161,23 +181,14 @@ __device__ __forceinline__ void load_geom_smem(const DevGeom* __restrict__ gp, D
     __syncthreads();
 }
 
-__device__ __forceinline__ void add_counters(unsigned long long* counters, unsigned long long c0,
-                                             unsigned long long c1, unsigned long long c2, unsigned long long c3,
-                                             unsigned long long c4) {
+// Adds the threads' work counts to the call's counters, one atomic per warp and count (a thread's own
+// counts fit 32 bits: it takes a share of at most 2^31 slots and stays far below that).
+__device__ __forceinline__ void add_counters(unsigned long long* counters, int c0, int c1, int c2, int c3, int c4) {
+    const int c[5] = {c0, c1, c2, c3, c4};
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        c0 += __shfl_xor_sync(kFull, c0, off);
-        c1 += __shfl_xor_sync(kFull, c1, off);
-        c2 += __shfl_xor_sync(kFull, c2, off);
-        c3 += __shfl_xor_sync(kFull, c3, off);
-        c4 += __shfl_xor_sync(kFull, c4, off);
-    }
-    if ((threadIdx.x & 31) == 0) {
-        if (c0) atomicAdd(counters + 0, c0);
-        if (c1) atomicAdd(counters + 1, c1);
-        if (c2) atomicAdd(counters + 2, c2);
-        if (c3) atomicAdd(counters + 3, c3);
-        if (c4) atomicAdd(counters + 4, c4);
+    for (int k = 0; k < 5; ++k) {
+        const long long sum = (long long)__reduce_add_sync(kFull, c[k]);
+        if ((threadIdx.x & 31) == 0 && sum) atomicAdd(counters + k, (unsigned long long)sum);
     }
 }
 
@@ -189,14 +200,31 @@ struct BuildArgs {
     BuildOutDev out;
     BuildWork w;
     unsigned long long* counters;
-    int max_steps;   // trail rows per seed (longest plan)
+    int slots;       // slots of the arrays (whole tiles)
     int nfound0;     // hits a track has when its search starts (3 seed hits forwards, 0 backwards)
-    int fused;       // 1: one k_round per plan step (per-round list lengths in w.rcounts)
 };
 
-// ---- round 0: slot 0 of every seed with work takes the seed state
-template <class F>
+// Child descriptor (one int4 per slot): parent slot | kind << 4 | disk << 8, the binned index of its
+// hit (K_HIT) or the seed (K_SEED), its score, its missed layers.  disk: the parent's prediction lies
+// on a disk.
+__device__ __forceinline__ int4 pack_child(int parent, int kind, bool disk, int q, float score, int nholes) {
+    return make_int4(parent | (kind << 4) | ((int)disk << 8), q, __float_as_int(score), nholes);
+}
+__device__ __forceinline__ int child_parent(const int4& d) { return d.x & 15; }
+__device__ __forceinline__ int child_kind(const int4& d) { return (d.x >> 4) & 15; }
+__device__ __forceinline__ int child_surface(const int4& d) {
+    return (d.x >> 8) & 1 ? MKGB_DISK : MKGB_BARREL;
+}
+
+template <class F> __device__ __forceinline__ const F* seed_states(const SeedStore& S) {
+    if constexpr (sizeof(F) == 4) return S.state;
+    else return S.state64;
+}
+
+// ---- round 0: the child in slot 0 of every seed with work is the seed itself
 __global__ void __launch_bounds__(kThreads) k_start(BuildArgs a) {
+    next_kernel_may_start();
+    wait_for_last_kernel();
     const DevGeom* __restrict__ g = a.geom;
     const int i = blockIdx.x * blockDim.x + threadIdx.x;   // seed position in the (event, eta, phi) order
     bool work = false;
@@ -217,1038 +245,508 @@ __global__ void __launch_bounds__(kThreads) k_start(BuildArgs a) {
         work = nsteps > 0;
         const int4 dead = make_int4(0, 0, 0, 0);
 #pragma unroll
-        for (int c = 1; c < kGroup; ++c) a.w.meta[0][i * kGroup + c] = dead;
-        if (work) {
-            const unsigned char* src = sizeof(F) == 4
-                ? reinterpret_cast<const unsigned char*>(a.S.state + (int64_t)seed * kSeedStateStride)
-                : reinterpret_cast<const unsigned char*>(a.S.state64 + (int64_t)seed * kSeedStateStride);
-            copy_state_rec<F>(src, a.w.st[0] + (int64_t)i * kGroup * state_bytes<F>());
-            a.w.meta[0][i * kGroup] = pack_meta(0.0f, 0.0f, a.nfound0, 0, false, true);
-        } else {
-            a.w.meta[0][i * kGroup] = dead;
-        }
+        for (int c = 1; c < kGroup; ++c) a.w.meta[0][slot_at(i * kGroup + c)] = dead;
+        a.w.meta[0][slot_at(i * kGroup)] = work ? pack_meta(0.0f, 0.0f, a.nfound0, 0, false, true) : dead;
+        if (work) a.w.child[slot_at(i * kGroup)] = pack_child(0, K_SEED, false, seed, 0.0f, 0);
     }
-    warp_append(work, i * kGroup, a.w.live[0], a.fused ? a.w.rcounts + 0 : a.w.counts + 0);
-    if (!a.fused) warp_append(work, i, a.w.seeds[0], a.w.counts + 2);
+    warp_append(work, i * kGroup, a.w.live[0], a.w.counts + 0);
+    warp_append(work, i, a.w.seeds[0], a.w.counts + 2);
 }
 
-// ---- a4-a9 for every live candidate of round tau
+// The update of a child redone in FP64 from its parent's FP32 prediction, narrowed (mixed
+// precision, growth G3).  False: the update failed.
+__device__ __noinline__ bool update_fp64(int surface, const Pred& pq, const float4* __restrict__ hb_pay, int hq,
+                                         State& t) {
+    PredT<double> qd;
+    qd.xh = pq.xh; qd.yh = pq.yh; qd.zh = pq.zh; qd.xl = pq.xl; qd.yl = pq.yl; qd.zl = pq.zl;
+    qd.k = pq.k; qd.phi = pq.phi; qd.th = pq.th; qd.tl = pq.tl; qd.pl = pq.pl;
+#pragma unroll
+    for (int q = 0; q < 15; ++q) qd.c[q] = pq.c[q];
+    double m[3], v[6];
+    load_hit(hb_pay, hq, m, v, nullptr);
+    StateT<double> td;
+    const bool ok = kalman_update(surface, qd, m[0], m[1], m[2], v, td);
+    if (ok) narrow_state(td, t);
+    return ok;
+}
 
-// MOD: module hits loaded (their chi2 on the module planes, the overlap bookkeeping); the plain
-// instantiation keeps the layers-only path's registers.
-template <class F, int TH, int MINB, bool BWD = false, bool MOD = false>
+// The state of a child from its record words f (its parent's prediction, or its own state for a
+// child that did not cross the parent's layer or is a seed).  Returns 0, 1 (the update failed) or 2
+// (an innovation covariance that FP32 cannot resolve: to be redone by update_fp64).
+template <class F>
+__device__ __forceinline__ int child_state(const BuildArgs& a, const int4& d, const F* f, const F m[3], const F v[6],
+                                           StateT<F>& t) {
+    const int kind = child_kind(d);
+    if (kind != K_HIT && kind != K_MISS) {
+        t.xh = f[0]; t.yh = f[1]; t.zh = f[2]; t.xl = f[3]; t.yl = f[4]; t.zl = f[5];
+        t.k = f[6]; t.phi = f[7]; t.th = f[8];
+#pragma unroll
+        for (int q = 0; q < 21; ++q) t.c[q] = f[9 + q];
+        t.tl = f[30];
+        t.pl = f[31];
+        return 0;
+    }
+    PredT<F> pq;
+    unpack_pred(f, pq);
+    const int surface = child_surface(d);
+    if (kind == K_HIT) {
+        float kap = 0.0f;
+        if (!kalman_update(surface, pq, m[0], m[1], m[2], v, t, &kap)) return 1;
+        return sizeof(F) == 4 && a.P.kappa_fp64 > 0.0f && kap > a.P.kappa_fp64 ? 2 : 0;
+    }
+    pred_to_state(surface, pq, t);
+    return 0;
+}
+
+// ---- a11 and a4-a7 for every live child of round tau: its state, then its way to the next layer
+
+// REDO: the children whose update the first launch left to FP64 (the
+// round's redo list).  BWD: the backward search (Sec. 2.2), crossing the layers behind the candidate.
+template <class F, int TH, int MINB, bool BWD = false, bool REDO = false>
+__global__ void __launch_bounds__(TH, MINB) k_move(BuildArgs a, int tau) {
+    __shared__ DevGeom g;
+    next_kernel_may_start();
+    if (!REDO) load_geom_smem(a.geom, g);
+    wait_for_last_kernel();
+    const int cur = tau & 1, nxt = cur ^ 1;
+    const int n = REDO ? a.w.counts[4] : a.w.counts[cur];
+    if (REDO) {
+        if (n == 0) return;
+        load_geom_smem(a.geom, g);
+    }
+    const int* __restrict__ list = REDO ? a.w.redo : a.w.live[cur];
+    if (!REDO && blockIdx.x == 0 && threadIdx.x == 0) {   // lists filled by this round's k_merge
+        a.w.counts[nxt] = 0;
+        a.w.counts[2 + nxt] = 0;
+    }
+    const DevParams& P = a.P;
+    const unsigned char* __restrict__ prev = a.w.rec[nxt];
+    unsigned char* __restrict__ rec = a.w.rec[cur];
+    int c_steps = 0, c_newton = 0, c_failed = 0;
+    const int stride = gridDim.x * TH;
+    // the descriptor of the next child is loaded one child ahead: it names the record to read
+    const int4 none = make_int4(0, 0, 0, 0);
+    const int first = blockIdx.x * TH + threadIdx.x;
+    int sl_next = first < n ? list[first] : 0;
+    int4 d_next = first < n ? a.w.child[slot_at(sl_next)] : none;
+    for (int base = blockIdx.x * TH; base < n; base += stride) {
+        // the warps of a block start a child together: they share the fetches of the loop's code
+        __syncthreads();
+        const int idx = base + threadIdx.x;
+        const int sl = sl_next;
+        const int4 d = d_next;
+        bool crossed = false;
+        int4 si = none;
+        StateT<F> t;
+        int fail = 4;   // no child
+        if (idx < n) {
+            si = a.w.sinfo[sl / kGroup];
+            F f[kStateWords];
+            F m[3] = {F(0), F(0), F(0)}, v[6] = {F(0), F(0), F(0), F(0), F(0), F(0)};
+            if (child_kind(d) == K_SEED)
+                load_seed_rec(seed_states<F>(a.S) + (int64_t)d.y * kSeedStateStride, f);
+            else
+                load_rec<F, kStateWords>(prev, (sl & ~(kGroup - 1)) | child_parent(d), f);
+            if (child_kind(d) == K_HIT) load_hit(a.H.hb_pay, d.y, m, v, nullptr);
+            if (idx + (int64_t)stride < n) {
+                sl_next = list[idx + stride];
+                d_next = a.w.child[slot_at(sl_next)];
+            }
+            if constexpr (REDO) {
+                Pred pq;
+                unpack_pred(f, pq);
+                fail = update_fp64(child_surface(d), pq, a.H.hb_pay, d.y, t) ? 0 : 3;
+            } else {
+                fail = child_state(a, d, f, m, v, t);
+            }
+        }
+        // children with and without a hit go on together (without this the compiler makes a copy of
+        // the rest for each kind: 17.7 of 32 lanes active instead of 28)
+        __syncwarp();
+        int nh_kind = K_NONE;
+        if (fail == 0) {
+            const DevLayer& L = g.layers[g.plan[si.x + tau]];
+            PredT<F> q;
+            F dir[4];
+            int newton = 0;
+            const int r = propagate_core<F, F, BWD>(L, g.cB, P.material, t, t.c, q, q.c, newton, dir);
+            c_newton += newton;
+            crossed = r > 0;
+            if (crossed) {
+                store_pred_rec(rec, sl, q, dir);
+                ++c_steps;
+            } else if (r == 0) {   // not crossed: the next child is this state
+                nh_kind = K_SKIP;
+                store_state_rec(rec, sl, t);
+            }
+        } else if (fail == 2) {   // redone in FP64 by the round's second launch
+            a.w.redo[atomicAdd(a.w.counts + 4, 1)] = sl;
+        } else if (fail != 4) {   // the child is dropped
+            a.w.meta[cur][slot_at(sl)].w = 0;
+            c_failed += fail == 1;
+        }
+        // (a crossed layer's list is k_find's)
+        if (!crossed && fail != 4) a.w.ls[word_at<2>(sl, 0)] = make_int4(0, nh_kind, d.z, 0);
+        warp_append(crossed, sl, a.w.found, a.w.counts + 5);
+    }
+    add_counters(a.counters, c_steps, 0, -c_failed, 0, c_newton);
+}
+
+// ---- a8-a9 for every candidate that crossed its layer in round tau
+//
+// Apart from k_move because the two want different things: this one waits for chains of small
+// loads (bin bounds, hits, their measurements) and needs many warps, that one computes and needs
+// registers.  It reads five of the record's eight words.
+template <class F, int TH, int MINB>
 __global__ void __launch_bounds__(TH, MINB) k_find(BuildArgs a, int tau) {
     __shared__ DevGeom g;
     // per-thread sorted list of hit children (chi2 asc, id asc), one column per thread
     __shared__ float s_x2[kGroup][TH];
     __shared__ int s_id[kGroup][TH];
     __shared__ int s_hq[kGroup][TH];
+    __shared__ int s_q[kQueue][TH];   // hits inside the window, waiting for their chi2
+    next_kernel_may_start();
     load_geom_smem(a.geom, g);
+    wait_for_last_kernel();
     const int tx = threadIdx.x;
-    const int cur = tau & 1, nxt = cur ^ 1;
-    if (blockIdx.x == 0 && threadIdx.x == 0) {   // lists filled by this round's k_select
-        a.w.counts[nxt] = 0;
-        a.w.counts[2 + nxt] = 0;
-        a.w.counts[4] = 0;
-    }
+    const int cur = tau & 1;
     const DevParams& P = a.P;
-    const int n = a.w.counts[cur];
-    const int* __restrict__ list = a.w.live[cur];
-    unsigned long long c_steps = 0, c_chi2 = 0, c_tested = 0, c_newton = 0;
-    const int stride = gridDim.x * blockDim.x;
-    // every lane of a warp runs the same number of iterations (warp_append inside k_select
-    // needs converged warps; here it keeps the loop uniform)
-    const int lane = threadIdx.x & 31;
-    // The next item's records (state, meta, seed info) are copied into this thread's column of
-    // s_rec while the current item is processed, so their load latency is hidden.  A column is
-    // read into registers before the next copy into it is issued (the copy's shared-memory write
-    // follows its global read, after these reads).  FP32 records and blocks of up to 128 threads
-    // only (static shared memory); the FP64 comparison path loads directly.
-    constexpr bool kPf = sizeof(F) == 4 && TH <= 128;
-    constexpr int kSW = kPf ? (int)(state_bytes<F>() / 16) : 1;   // 16-byte words of a state record
-    __shared__ int4 s_rec[kSW + 2][kPf ? TH : 1];
-    auto fetch = [&](int slot) {
-        const int4* src = reinterpret_cast<const int4*>(a.w.st[cur] + (int64_t)slot * state_bytes<F>());
-#pragma unroll
-        for (int j = 0; j < kSW; ++j) cp_async16(&s_rec[j][tx], src + j);
-        cp_async16(&s_rec[kSW][tx], a.w.meta[cur] + slot);
-        cp_async16(&s_rec[kSW + 1][tx], a.w.sinfo + slot / kGroup);
-    };
-    int sl_cur = -1, sl_next = -1;
-    {
-        const int first = blockIdx.x * blockDim.x + (threadIdx.x & ~31) + lane;
-        sl_cur = first < n ? list[first] : -1;
-        if constexpr (kPf) {
-            if (sl_cur >= 0) fetch(sl_cur);
-            cp_async_commit();
-        }
-        if (first + stride < n) sl_next = list[first + stride];
-    }
-    for (int base = blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < n; base += stride) {
-        const int idx = base + lane;
-        const int sl = sl_cur;
-        int4 si = make_int4(0, 0, 0, 0), mt = make_int4(0, 0, 0, 0);
-        StateT<F> t;
-        if constexpr (kPf) {
-            cp_async_wait_all();
-            if (sl >= 0) {
-                si = s_rec[kSW + 1][tx];
-                mt = s_rec[kSW][tx];
-                F f[32];
-#pragma unroll
-                for (int j = 0; j < kSW; ++j)
-                    unpack16(*reinterpret_cast<const typename Vec16<F>::T*>(&s_rec[j][tx]), f + j * (16 / sizeof(F)));
-                t.xh = f[0]; t.yh = f[1]; t.zh = f[2]; t.xl = f[3]; t.yl = f[4]; t.zl = f[5];
-                t.k = f[6]; t.phi = f[7]; t.th = f[8];
-#pragma unroll
-                for (int q = 0; q < 21; ++q) t.c[q] = f[9 + q];
-                t.tl = f[30];
-                t.pl = f[31];
-            }
-            asm volatile("" ::: "memory");
-            sl_cur = sl_next;
-            if (sl_cur >= 0) fetch(sl_cur);
-            cp_async_commit();
-        } else {
-            if (sl >= 0) {
-                si = a.w.sinfo[sl / kGroup];
-                mt = a.w.meta[cur][sl];
-                load_state_rec(a.w.st[cur] + (int64_t)sl * state_bytes<F>(), t);
-            }
-            sl_cur = sl_next;
-        }
-        sl_next = idx + 2 * stride < n ? list[idx + 2 * stride] : -1;
-        if (idx >= n) continue;
-        const int layer = g.plan[si.x + tau];
-        const DevLayer& L = g.layers[layer];
-        if (mt.w == 0) {   // dropped after the selection (its FP64 update redo failed)
-            a.w.ls[(int64_t)sl * 5] = make_int4(0, K_NONE, 0, 0);
-            continue;
-        }
-        const float score = __int_as_float(mt.x);
-        const int nholes = (mt.z >> 8) & 0xff;
-
+    const int n = a.w.counts[5];
+    int c_chi2 = 0, c_tested = 0;
+    const int stride = gridDim.x * TH;
+    for (int idx = blockIdx.x * TH + tx; idx < n; idx += stride) {
+        const int sl = a.w.found[idx];
+        const int4 d = a.w.child[slot_at(sl)];
+        const int4 si = a.w.sinfo[sl / kGroup];
         PredT<F> q;
         F dir[4];
-        int newton = 0;
-        // BWD: the backward search (Sec. 2.2), crossing the plan's layers behind the candidate
-        const int r = propagate_core<F, F, BWD>(L, g.cB, P.material, t, t.c, q, q.c, newton, dir);
-        c_newton += newton;
-        int nh_kind = K_NONE, n_h = 0;
-        float nh_score = 0.0f;
-        // overlap pickup (Sec. 2.2): the best accepted module hit b1 (the list's first entry on a
-        // modular layer) and the best one on another module b2 (binned index, -1 none)
-        int b1m = -1, b2 = -1, b2id = 0;
-        float b1x = 0.0f, b2x = 0.0f;
-        int b1id = 0, b1q = -1;
-        if (r == 0) {
-            nh_kind = K_SKIP;
-            nh_score = score;
-        } else if (r > 0) {
-            ++c_steps;
-            if (nholes < P.max_holes) {
-                nh_kind = K_MISS;
-                nh_score = score - P.score_hole;
-            } else {
-                nh_kind = K_STOP;
-                nh_score = score;
-            }
-            const FrameT<F> fr = frame_of(L.kind, q.xh, q.yh, dir[0], dir[1], dir[2], dir[3]);
-            const WindowT<F> w = window(L, P, q, fr);
-            const float eps = 1e-5f;
-            const float fe0 = (w.eta - w.deta - eps - L.eta_lo) * L.eta_scale;
-            const float fe1 = (w.eta + w.deta + eps - L.eta_lo) * L.eta_scale;
-            const int e0 = fe0 >= 0.0f ? (int)fminf(floorf(fe0), (float)(L.n_eta - 1)) : 0;
-            const int e1 = fe1 >= 0.0f ? (int)fminf(floorf(fe1), (float)(L.n_eta - 1)) : 0;
-            const float pscale = L.n_phi * (1.0f / kTwoPi);
-            const int f0 = (int)floorf((w.phi - w.dphi - eps + kPi) * pscale);
-            const int f1 = (int)floorf((w.phi + w.dphi + eps + kPi) * pscale);
-            int nf = f1 - f0 + 1;
-            int fa = f0 % L.n_phi;
-            if (fa < 0) fa += L.n_phi;
-            if (nf >= L.n_phi) {
-                nf = L.n_phi;
-                fa = 0;
-            }
-            const int run1 = min(nf, L.n_phi - fa), run2 = nf - run1;
-            const int64_t bb = (int64_t)si.w * g.bins_per_event + L.bin_base;
-            for (int ie = e0; ie <= e1; ++ie) {
-                const int64_t rowb = bb + (int64_t)ie * L.n_phi;
-                for (int run = 0; run < 2; ++run) {
-                    const int b0 = run == 0 ? fa : 0;
-                    const int nb = run == 0 ? run1 : run2;
-                    if (nb <= 0) continue;
-                    const int q0 = __ldg(a.H.bin_start + rowb + b0);
-                    const int q1 = __ldg(a.H.bin_start + rowb + b0 + nb);
-                    for (int hq = q0; hq < q1; ++hq) {
-                        ++c_tested;
-                        const float2 ep = __ldg(a.H.hb_ep + hq);
-                        if (fabs(F(ep.x) - w.eta) <= w.deta && fabs(wrap_pi(F(ep.y) - w.phi)) <= w.dphi) {
-                            ++c_chi2;
-                            F m[3], v[6];
-                            int id, md = -1;
-                            F x2f;
-                            bool okx;
-                            if constexpr (MOD) {
-                                load_hit(a.H.hb_pay, hq, m, v, &id, &md);
-                                // a module hit: chi2 on its module's plane (Sec. 3.1)
-                                okx = md >= 0 ? module_chi2_dir(q, fr, dir, g.mods, md, g.cB, m, v, x2f)
-                                              : chi2_hit(fr, q, m[0], m[1], m[2], v, x2f);
-                            } else {
-                                load_hit(a.H.hb_pay, hq, m, v, &id);
-                                okx = chi2_hit(fr, q, m[0], m[1], m[2], v, x2f);
-                            }
-                            if (okx && x2f < F(P.chi2_cut)) {
-                                const float x2 = float(x2f);   // scores and child order in FP32
-                                if (MOD && md >= 0) {
-                                    if (b1m < 0 || x2 < b1x || (x2 == b1x && id < b1id)) {
-                                        if (b1m >= 0 && md != b1m) {   // the previous b1 becomes b2
-                                            b2 = b1q; b2x = b1x; b2id = b1id;
-                                        }
-                                        b1q = hq; b1x = x2; b1id = id; b1m = md;
-                                    } else if (md != b1m && (b2 < 0 || x2 < b2x || (x2 == b2x && id < b2id))) {
-                                        b2 = hq; b2x = x2; b2id = id;
-                                    }
-                                }
-                                // insert into the sorted list (kept to its first kGroup entries)
-                                int j = n_h < kGroup ? n_h : kGroup - 1;
-                                const bool fits = n_h < kGroup ||
-                                                  x2 < s_x2[j][tx] || (x2 == s_x2[j][tx] && id < s_id[j][tx]);
-                                if (fits) {
-                                    while (j > 0 && (x2 < s_x2[j - 1][tx] ||
-                                                     (x2 == s_x2[j - 1][tx] && id < s_id[j - 1][tx]))) {
-                                        s_x2[j][tx] = s_x2[j - 1][tx];
-                                        s_id[j][tx] = s_id[j - 1][tx];
-                                        s_hq[j][tx] = s_hq[j - 1][tx];
-                                        --j;
-                                    }
-                                    s_x2[j][tx] = x2;
-                                    s_id[j][tx] = id;
-                                    s_hq[j][tx] = hq;
-                                    if (n_h < kGroup) ++n_h;
-                                }
-                            }
-                        }
-                    }
-                }
-            }
-            store_pred_rec(a.w.pr + (int64_t)sl * pred_bytes<F>(), q);
+        load_pred_rec(a.w.rec[cur], sl, q, dir);
+        const DevLayer& L = g.layers[g.plan[si.x + tau]];
+        const float score = __int_as_float(d.z);
+        const bool miss = d.w < P.max_holes;
+        const int nh_kind = miss ? K_MISS : K_STOP;
+        const float nh_score = miss ? score - P.score_hole : score;
+        int n_h = 0;
+        const FrameT<F> fr = frame_of(L.kind, q.xh, q.yh, dir[0], dir[1], dir[2], dir[3]);
+        const WindowT<F> w = window(L, P, q, fr);
+        const float eps = 1e-5f;
+        const float fe0 = (w.eta - w.deta - eps - L.eta_lo) * L.eta_scale;
+        const float fe1 = (w.eta + w.deta + eps - L.eta_lo) * L.eta_scale;
+        const int e0 = fe0 >= 0.0f ? (int)fminf(floorf(fe0), (float)(L.n_eta - 1)) : 0;
+        const int e1 = fe1 >= 0.0f ? (int)fminf(floorf(fe1), (float)(L.n_eta - 1)) : 0;
+        const float pscale = L.n_phi * (1.0f / kTwoPi);
+        const int f0 = (int)floorf((w.phi - w.dphi - eps + kPi) * pscale);
+        const int f1 = (int)floorf((w.phi + w.dphi + eps + kPi) * pscale);
+        int nf = f1 - f0 + 1;
+        int fa = f0 % L.n_phi;
+        if (fa < 0) fa += L.n_phi;
+        if (nf >= L.n_phi) {
+            nf = L.n_phi;
+            fa = 0;
         }
-        int4* lrec = a.w.ls + (int64_t)sl * 5;
-        lrec[0] = make_int4(n_h, nh_kind, __float_as_int(nh_score), MOD ? b2 : -1);
-        for (int j = 0; j < n_h; j += 2)
-            lrec[1 + j / 2] = make_int4(__float_as_int(s_x2[j][tx]), s_hq[j][tx],
-                                        __float_as_int(j + 1 < n_h ? s_x2[j + 1][tx] : kBig),
-                                        j + 1 < n_h ? s_hq[j + 1][tx] : 0);
+        const int run1 = min(nf, L.n_phi - fa), run2 = nf - run1;
+        const int64_t bb = (int64_t)si.w * g.bins_per_event + L.bin_base;
+        // the window's bins are ranges of hits, one or two (around phi = pi) per eta row; the bounds
+        // of the next range are loaded while the hits of this one are tested, two at a time, and
+        // the hits inside the window are queued, so that the lanes of a warp meet at the chi2
+        const int nr = run2 > 0 ? 2 : 1, n_ranges = (e1 - e0 + 1) * nr;
+        auto bounds = [&](int rg, int& q0, int& q1) {
+            const int64_t at = bb + (int64_t)(e0 + (rg >> (nr - 1))) * L.n_phi + ((rg & (nr - 1)) ? 0 : fa);
+            q0 = __ldg(a.H.bin_start + at);
+            q1 = __ldg(a.H.bin_start + at + ((rg & (nr - 1)) ? run2 : run1));
+        };
+        auto inside = [&](const float2& ep) {
+            return fabs(F(ep.x) - w.eta) <= w.deta && fabs(wrap_pi(F(ep.y) - w.phi)) <= w.dphi;
+        };
+        int rg = 0, hq = 0, q1 = 0, hq_next = 0, q1_next = 0;
+        if (n_ranges > 0) bounds(0, hq_next, q1_next);
+        for (bool more = true; more;) {
+            int nq = 0;
+            while (nq < kQueue) {
+                if (hq >= q1) {
+                    if (rg >= n_ranges) {
+                        more = false;
+                        break;
+                    }
+                    hq = hq_next;
+                    q1 = q1_next;
+                    if (++rg < n_ranges) bounds(rg, hq_next, q1_next);
+                    continue;
+                }
+                const bool two = hq + 1 < q1 && nq + 1 < kQueue;
+                const float2 ep0 = __ldg(a.H.hb_ep + hq), ep1 = __ldg(a.H.hb_ep + hq + (int)two);
+                c_tested += 1 + two;
+                if (inside(ep0)) s_q[nq++][tx] = hq;
+                if (two && inside(ep1)) s_q[nq++][tx] = hq + 1;
+                hq += 1 + two;
+            }
+            c_chi2 += nq;
+            for (int jq = 0; jq < nq; ++jq) {
+                const int h = s_q[jq][tx];
+                F mh[3], vh[6];
+                int id;
+                F x2f;
+                load_hit(a.H.hb_pay, h, mh, vh, &id);
+                const bool okx = chi2_hit(fr, q, mh[0], mh[1], mh[2], vh, x2f);
+                if (!okx || !(x2f < F(P.chi2_cut))) continue;
+                const float x2 = float(x2f);   // scores and child order in FP32
+                // insert into the sorted list (kept to its first kGroup entries)
+                int j = n_h < kGroup ? n_h : kGroup - 1;
+                if (n_h == kGroup && !(x2 < s_x2[j][tx] || (x2 == s_x2[j][tx] && id < s_id[j][tx]))) continue;
+                while (j > 0 && (x2 < s_x2[j - 1][tx] || (x2 == s_x2[j - 1][tx] && id < s_id[j - 1][tx]))) {
+                    s_x2[j][tx] = s_x2[j - 1][tx];
+                    s_id[j][tx] = s_id[j - 1][tx];
+                    s_hq[j][tx] = s_hq[j - 1][tx];
+                    --j;
+                }
+                s_x2[j][tx] = x2;
+                s_id[j][tx] = id;
+                s_hq[j][tx] = h;
+                if (n_h < kGroup) ++n_h;
+            }
+        }
+        // the child list: its header and first two hits, the other hits apart
+        int4* lrec = a.w.ls + word_at<2>(sl, 0);
+        lrec[0] = make_int4(n_h | (L.kind == MKGB_DISK ? kDiskBit : 0), nh_kind, __float_as_int(nh_score), 0);
+        for (int j = 0; j < n_h; j += 2) {
+            const int4 e = make_int4(__float_as_int(s_x2[j][tx]), s_hq[j][tx],
+                                     __float_as_int(j + 1 < n_h ? s_x2[j + 1][tx] : kBig),
+                                     j + 1 < n_h ? s_hq[j + 1][tx] : 0);
+            if (j == 0)
+                lrec[kTile * kGroup] = e;
+            else
+                a.w.ls_more[word_at<3>(sl, j / 2 - 1)] = e;
+        }
     }
-    add_counters(a.counters, c_steps, c_chi2, 0ull, c_tested, c_newton);
+    add_counters(a.counters, 0, c_chi2, 0, c_tested, 0);
 }
 
-// ---- a10-a11 for every seed with a live candidate in round tau
-template <class F, int TH, int MINB, bool MOD = false>
-__global__ void __launch_bounds__(TH, MINB) k_select(BuildArgs a, int tau) {
-    __shared__ DevGeom g;
-    load_geom_smem(a.geom, g);
+// ---- a10 for every seed with a live candidate in round tau
+//
+// Eight lanes per seed, lane = parent slot.  Every child of the seed puts its key (score, then parent
+// slot, then place in the parent's list) into shared memory and counts the keys above its own: that
+// count is its slot among the N best, so a parent's lane writes its kept children straight from its
+// registers, with no exchange of their contents and no round per rank. 
+// 64 events: 4.8 ms; eight lanes exchanging keys and contents by shuffles, a round per rank: 7.4 ms;
+// one thread per seed with its eight best in registers: 3.8 ms, but 1.3 times the whole search of one
+// event (0.86 against 0.66 ms), where the latency of a thread's serial lists counts.
+constexpr int kNoHit = 15;   // place of the child without a hit
+constexpr int kSeedKeys = kGroup * (kGroup + 1);
+__device__ __forceinline__ unsigned long long child_key(float score, int slot, int place) {
+    unsigned u = __float_as_uint(score);
+    u = (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+    return ((unsigned long long)u << 32) | (unsigned)(0xffff - (slot << 4 | place));
+}
+
+template <class F, int TH, int MINB>
+__global__ void __launch_bounds__(TH, MINB) k_merge(BuildArgs a, int tau) {
+    __shared__ unsigned long long s_key[TH / kGroup][kSeedKeys];
+    __shared__ int s_cnt[2][TH / 32], s_base[2];
+    next_kernel_may_start();
+    wait_for_last_kernel();
     const int cur = tau & 1, nxt = cur ^ 1;
     const DevParams& P = a.P;
-    const int lane = threadIdx.x & 31;
-    const int slot = lane & 7, gbase = lane & ~7;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, slot = lane & 7, gbase = lane & ~7;
+    unsigned long long* keys = s_key[threadIdx.x / kGroup];
     const int n = a.w.counts[2 + cur];
     const int* __restrict__ list = a.w.seeds[cur];
-    unsigned long long c_upd = 0;
-    const int groups_per_block = TH / kGroup;
-    const int gstride = gridDim.x * groups_per_block;
-    // loop bound uniform over the warp: the first group index of the warp
-    const int g0 = blockIdx.x * groups_per_block + (threadIdx.x >> 5) * 4;
-    for (int wg = g0; wg < n; wg += gstride) {
-        const int gi = wg + (lane >> 3);
+    if (blockIdx.x == 0 && threadIdx.x == 0) {   // the redo list and k_find's list of the next round
+        a.w.counts[4] = 0;
+        a.w.counts[5] = 0;
+    }
+    int c_upd = 0;
+    const int gstride = gridDim.x * (TH / kGroup);
+    for (int bg = blockIdx.x * (TH / kGroup); bg < n; bg += gstride) {   // uniform over the block
+        const int gi = bg + wid * 4 + (lane >> 3);
         const bool gact = gi < n;
-        const int i = gact ? list[gi] : 0;
-        const int4 si = gact ? a.w.sinfo[i] : make_int4(0, 0, 0, 0);
+        const int i = list[gact ? gi : bg];
+        const int nsteps = a.w.sinfo[i].z;
         const int sl = i * kGroup + slot;
-        const int4 mt = gact ? a.w.meta[cur][sl] : make_int4(0, 0, 0, 0);
+        // all of the slot's words at once (those of an empty slot are not used)
+        const int4 mt = a.w.meta[cur][slot_at(sl)];
+        const int4 e0 = a.w.ls[word_at<2>(sl, 0)], e1 = a.w.ls[word_at<2>(sl, 1)];
         const float score = __int_as_float(mt.x);
-        const bool alive = mt.w != 0;
-        const bool stopped = ((mt.z >> 16) & 1) != 0;
+        const bool alive = gact && mt.w != 0, stopped = ((mt.z >> 16) & 1) != 0;
+        const bool searched = alive && !stopped;
+        const int n_h = searched ? e0.x & (kDiskBit - 1) : 0;
+        const int nh_kind = !alive ? K_NONE : stopped ? K_CARRY : e0.y;
+        const float nh_score = stopped ? score : __int_as_float(e0.z);
+        const bool disk = (e0.x & kDiskBit) != 0;
+        const bool has_nh = nh_kind != K_NONE;
+        auto hit_entry = [&](int j) {   // (chi2, binned index) of the parent's j-th hit
+            if (j == 0) return make_int2(e1.x, e1.y);
+            if (j == 1) return make_int2(e1.z, e1.w);
+            return reinterpret_cast<const int2*>(a.w.ls_more + word_at<3>(sl, j / 2 - 1))[j & 1];
+        };
+        auto hit_score = [&](int j) { return score + P.score_hit - __int_as_float(hit_entry(j).x); };
 
-        int nh_kind = K_NONE;
-        float nh_score = -kBig;
-        int b1q = -1, b2q = -1;   // the parent's best module hit and best hit on another module
-        float lx[kGroup];
-        int lq[kGroup];
+        // ---- the seed's children and the slots they take
+        const int cnt = n_h + (int)has_nh;
+        int end = cnt;
 #pragma unroll
-        for (int j = 0; j < kGroup; ++j) {
-            lx[j] = kBig;
-            lq[j] = 0;
+        for (int d = 1; d < kGroup; d <<= 1) {
+            const int o = __shfl_up_sync(kFull, end, d, kGroup);
+            if (slot >= d) end += o;
         }
-        if (alive) {
-            if (stopped) {
-                nh_kind = K_CARRY;
-                nh_score = score;
-            } else {
-                const int4* lrec = a.w.ls + (int64_t)sl * 5;
-                int4 e[5];
-#pragma unroll
-                for (int q = 0; q < 5; ++q) e[q] = lrec[q];   // all at once; entries past the count unused
-                nh_kind = e[0].y;
-                nh_score = __int_as_float(e[0].z);
-#pragma unroll
-                for (int j = 0; j < kGroup; j += 2) {
-                    if (j < e[0].x) {
-                        lx[j] = __int_as_float(e[1 + j / 2].x);
-                        lq[j] = e[1 + j / 2].y;
-                    }
-                    if (j + 1 < e[0].x) {
-                        lx[j + 1] = __int_as_float(e[1 + j / 2].z);
-                        lq[j + 1] = e[1 + j / 2].w;
-                    }
-                }
-                if constexpr (MOD) {
-                    b2q = e[0].w;
-                    b1q = e[0].x > 0 ? lq[0] : -1;
-                }
-            }
+        const int total = __shfl_sync(kFull, end, kGroup - 1, kGroup);
+        for (int j = 0; j < n_h; ++j) keys[end - cnt + j] = child_key(hit_score(j), slot, j);
+        if (has_nh) keys[end - 1] = child_key(nh_score, slot, kNoHit);
+        __syncwarp();
+        auto rank_of = [&](unsigned long long k) {
+            int r = 0;
+            for (int q = 0; q < total; ++q) r += keys[q] > k;
+            return r;
+        };
+        int kept_hits = 0;         // the first of the parent's hits are kept, at these slots (4 bits each)
+        unsigned hit_slots = 0, kept = 0, live = 0;
+        for (int j = 0; j < n_h; ++j) {
+            const int r = rank_of(keys[end - cnt + j]);
+            if (r >= P.max_cands) break;   // the others come after it
+            hit_slots |= (unsigned)r << (4 * j);
+            live |= 1u << r;
+            ++kept_hits;
         }
-        // a parent whose accepted module hits span two modules gives every hit child an overlap
-        // hit (Sec. 2.2) and its score
-        const float ovl_bonus = MOD && b2q >= 0 ? P.score_overlap : 0.0f;
-
-        // ---- the N best children of the seed (a10)
-        bool nh_avail = nh_kind != K_NONE;
-        int my_parent = -1, my_kind = K_NONE, my_q = 0, my_b1 = -1, my_b2 = -1;
-        float my_x2 = 0.0f, my_score = 0.0f;
-        for (int r = 0; r < P.max_cands; ++r) {
-            const bool has_hit = lx[0] < kBig;
-            float hit_score = score + P.score_hit - lx[0];
-            if constexpr (MOD) hit_score += ovl_bonus;
-            int hk = K_NONE;
-            float hs = 0.0f;
-            if (has_hit && (!nh_avail || hit_score >= nh_score)) {
-                hk = K_HIT;
-                hs = hit_score;
-            } else if (nh_avail) {
-                hk = nh_kind;
-                hs = nh_score;
-            }
-            unsigned long long best = hk != K_NONE ? order_key(hs, slot) : 0ull;
+        c_upd += kept_hits;
+        const int nh_slot = has_nh ? rank_of(keys[end - 1]) : kGroup;
+        const bool nh_kept = nh_slot < P.max_cands && has_nh;
+        const bool nh_stop = nh_kept && nh_kind == K_STOP;
+        kept = live | (nh_kept ? 1u << nh_slot : 0u);
+        if (nh_kept && (nh_kind == K_MISS || nh_kind == K_SKIP)) live |= 1u << nh_slot;
+        const bool more = gact && tau + 1 < nsteps;
+        const unsigned used = nh_kept && nh_kind == K_CARRY ? 1u << ((mt.z >> 18) & 7) : 0u;   // stop records in use
+        const unsigned all_kept = __reduce_or_sync(kFull, kept << gbase);
+        const unsigned all_live = __reduce_or_sync(kFull, more ? live << gbase : 0u);
+        const unsigned all_used = __reduce_or_sync(kFull, used << gbase);
+        const unsigned all_stop = __ballot_sync(kFull, nh_stop);   // (also the end of the keys' use)
+        const unsigned seed_kept = (all_kept >> gbase) & 0xffu;
+        const bool p_seed = more && seed_kept != 0 && slot == 0;
+        const unsigned ms = __ballot_sync(kFull, p_seed);
+        if (lane == 0) {
+            s_cnt[0][wid] = __popc(all_live);
+            s_cnt[1][wid] = __popc(ms);
+        }
+        __syncthreads();
+        int bl = 0, bs = 0, tl = 0, ts = 0;
 #pragma unroll
-            for (int off = 1; off < kGroup; off <<= 1) {
-                const unsigned long long o = __shfl_xor_sync(kFull, best, off);
-                best = o > best ? o : best;
-            }
-            const bool valid = best != 0ull;
-            const int wslot = kGroup - 1 - (int)(best & 7ull);
-            const int src = gbase + wslot;
-            const int w_kind = shfl_i(hk, src);
-            const int w_q = shfl_i(lq[0], src);
-            const float w_x2 = shfl_f(lx[0], src);
-            const float w_score = shfl_f(hs, src);
-            if (valid && slot == r) {
-                my_parent = wslot;
-                my_kind = w_kind;
-                my_q = w_q;
-                my_x2 = w_x2;
-                my_score = w_score;
-            }
-            if constexpr (MOD) {
-                const int w_b1 = shfl_i(b1q, src), w_b2 = shfl_i(b2q, src);
-                if (valid && slot == r) {
-                    my_b1 = w_b1;
-                    my_b2 = w_b2;
-                }
-            }
-            if (valid && slot == wslot) {
-                if (hk == K_HIT) {
-#pragma unroll
-                    for (int j = 0; j < kGroup - 1; ++j) {
-                        lx[j] = lx[j + 1];
-                        lq[j] = lq[j + 1];
-                    }
-                    lx[kGroup - 1] = kBig;
-                } else {
-                    nh_avail = false;
-                }
-            }
+        for (int q = 0; q < TH / 32; ++q) {
+            bl += q < wid ? s_cnt[0][q] : 0;
+            bs += q < wid ? s_cnt[1][q] : 0;
+            tl += s_cnt[0][q];
+            ts += s_cnt[1][q];
+        }
+        if (threadIdx.x == 0) {   // the block's two list reservations, in flight during the writes below
+            s_base[0] = tl ? atomicAdd(a.w.counts + nxt, tl) : 0;
+            s_base[1] = ts ? atomicAdd(a.w.counts + 2 + nxt, ts) : 0;
         }
 
-        // ---- the child's state (a11), meta, trail and next-round lists
-        const int psrc = gbase + (my_parent >= 0 ? my_parent : slot);
-        const int4 pm = make_int4(shfl_i(mt.x, psrc), shfl_i(mt.y, psrc), shfl_i(mt.z, psrc), shfl_i(mt.w, psrc));
-        bool c_alive = false, c_stopped = false;
-        float chi2s = __int_as_float(pm.y);
-        int nfound = pm.z & 0xff, nholes = (pm.z >> 8) & 0xff;
-        int code = MKGB_HIT_STOP;
-        const int csl = i * kGroup + slot;
-        bool rescue = false;
-        int ovl = -1;
-        if (gact && my_kind != K_NONE) {
-            const int psl = i * kGroup + my_parent;
-            c_alive = true;
-            c_stopped = ((pm.z >> 16) & 1) != 0;
-            if (my_kind == K_SKIP || my_kind == K_CARRY) {
-                copy_state_rec<F>(a.w.st[cur] + (int64_t)psl * state_bytes<F>(),
-                                  a.w.st[nxt] + (int64_t)csl * state_bytes<F>());
-                if (my_kind == K_SKIP) code = MKGB_HIT_SKIP;
-            } else {
-                const DevLayer& L = g.layers[g.plan[si.x + tau]];
-                PredT<F> pq;
-                load_pred_rec(a.w.pr + (int64_t)psl * pred_bytes<F>(), pq);
-                StateT<F> t;
-                if (my_kind == K_HIT) {
-                    F m[3], v[6];
-                    int id, md = -1;
-                    if constexpr (MOD)
-                        load_hit(a.H.hb_pay, my_q, m, v, &id, &md);
-                    else
-                        load_hit(a.H.hb_pay, my_q, m, v, &id);
-                    float kap = 0.0f;
-                    bool ok;
-                    if (MOD && md >= 0) {   // a module hit: the update on its module's plane (Sec. 3.1)
-                        F x2u;
-                        ok = module_update(L.kind, pq, g.mods, md, g.cB, m, v, 0.0f, t, x2u, kap) == 0;
-                        if (my_b2 >= 0) {   // the overlap hit: b1 unless the hit is on b1's module
-                            const int m1 = __float_as_int(__ldg(a.H.hb_pay + 3 * (int64_t)my_b1 + 2).z);
-                            const int oq = md != m1 ? my_b1 : my_b2;
-                            ovl = __float_as_int(__ldg(a.H.hb_pay + 3 * (int64_t)oq).w);
-                        }
-                    } else {
-                        ok = kalman_update(L.kind, pq, m[0], m[1], m[2], v, t, &kap);
-                    }
-                    if (ok) {
-                        chi2s += my_x2;
-                        ++nfound;
-                        ++c_upd;
-                        code = id;
-                        // FP32 cannot resolve an innovation covariance this ill-conditioned: the
-                        // update is redone in FP64 by k_rescue (mixed precision, growth G3)
-                        rescue = sizeof(F) == 4 && P.kappa_fp64 > 0.0f && kap > P.kappa_fp64;
-                    } else {
-                        c_alive = false;
-                    }
-                } else {
-                    pred_to_state(L.kind, pq, t);
-                    if (my_kind == K_MISS) {
-                        ++nholes;
-                        code = MKGB_HIT_MISS;
-                    } else {   // K_STOP
-                        c_stopped = true;
-                    }
-                }
-                store_state_rec(a.w.st[nxt] + (int64_t)csl * state_bytes<F>(), t);
+        // ---- the kept children: descriptors, meta, trail
+        auto put = [&](int r, int kind, float child_score, int4 cm, int code, int hq) {
+            const int cs = i * kGroup + r;
+            const int at = slot_at(cs);
+            a.w.child[at] = pack_child(slot, kind, disk, hq, child_score, (cm.z >> 8) & 0xff);
+            a.w.meta[nxt][at] = cm;
+            a.w.trail[(int64_t)tau * a.slots + at] = ((code + 4) << 3) | slot;
+        };
+        const float chi2s = __int_as_float(mt.y);
+        const int nfound = mt.z & 0xff, nholes = (mt.z >> 8) & 0xff;
+        for (int j = 0; j < kept_hits; ++j) {   // (a child whose update fails is dropped by the next k_move)
+            const int2 e = hit_entry(j);
+            const float sc = hit_score(j);
+            put((hit_slots >> (4 * j)) & 15, K_HIT, sc,
+                pack_meta(sc, chi2s + __int_as_float(e.x), nfound + 1, nholes, false, true), e.y, e.y);
+        }
+        if (nh_kept) {
+            const bool stop = nh_kind == K_STOP || nh_kind == K_CARRY;
+            int4 cm = pack_meta(nh_score, chi2s, nfound, nholes + (nh_kind == K_MISS), stop, true);
+            if (nh_kind == K_CARRY) cm.z |= mt.z & (15 << 17);
+            if (nh_kind == K_STOP) {   // the prediction where it stopped is put aside for the search's end
+                unsigned free = ~(all_used >> gbase) & 0xffu;
+                for (int q = __popc((all_stop >> gbase) & ((1u << slot) - 1u)); q > 0; --q) free &= free - 1;
+                const int k = __ffs(free) - 1;
+                cm.z |= ((int)disk << 17) | (k << 18);
+                F f[kPredWords];
+                load_rec<F, kPredWords>(a.w.rec[cur], sl, f);
+                store_rec<F, kPredWords>(a.w.stop, i * kGroup + k, f);
             }
-            a.w.trail[((int64_t)i * a.max_steps + tau) * kGroup + slot] = ((code + 4) << 3) | my_parent;
-            if (MOD && a.w.otrail) a.w.otrail[((int64_t)i * a.max_steps + tau) * kGroup + slot] = c_alive ? ovl : -1;
+            put(nh_slot, nh_kind, nh_score, cm,
+                nh_kind == K_MISS ? MKGB_HIT_MISS : nh_kind == K_SKIP ? MKGB_HIT_SKIP : MKGB_HIT_STOP, 0);
         }
-        const bool more = gact && tau + 1 < si.z;
-        const unsigned am = __ballot_sync(kFull, c_alive);
-        const bool any = ((am >> gbase) & 0xffu) != 0u;
-        const bool p_live = more && c_alive && !c_stopped, p_seed = more && any && slot == 0;
-        const unsigned m0 = __ballot_sync(kFull, rescue), m1 = __ballot_sync(kFull, p_live),
-                       m2 = __ballot_sync(kFull, p_seed);
-        int b0 = 0, b1 = 0, b2 = 0;
-        if (lane == 0) {   // the three list reservations of the warp, in flight together
-            if (m0) b0 = atomicAdd(a.w.counts + 4, __popc(m0));
-            if (m1) b1 = atomicAdd(a.w.counts + nxt, __popc(m1));
-            if (m2) b2 = atomicAdd(a.w.counts + 2 + nxt, __popc(m2));
-        }
-        if (gact) a.w.meta[nxt][csl] = pack_meta(my_score, chi2s, nfound, nholes, c_stopped, c_alive);
-        if (gact && slot == 0 && (!more || !any)) a.w.fin[i] = nxt | ((tau + 1) << 1);
-        b0 = __shfl_sync(kFull, b0, 0);
-        b1 = __shfl_sync(kFull, b1, 0);
-        b2 = __shfl_sync(kFull, b2, 0);
+        if (gact && !((seed_kept >> slot) & 1)) a.w.meta[nxt][slot_at(sl)] = make_int4(0, 0, 0, 0);
+        if (gact && slot == 0 && !p_seed) a.w.fin[i] = tau + 1;
+
+        // ---- next-round lists, in the seeds' and slots' order: a block's 32 seeds stay together, or the
+        // lists, and with them the tiles that a warp of the next round touches, would come apart in
+        // pieces of a warp's four seeds (27.6 ms per 64-event search)
+        __syncthreads();
         const unsigned below = (1u << lane) - 1u;
-        if (rescue) a.w.rescue[b0 + __popc(m0 & below)] = csl;
-        if (p_live) a.w.live[nxt][b1 + __popc(m1 & below)] = csl;
-        if (p_seed) a.w.seeds[nxt][b2 + __popc(m2 & below)] = i;
+        if ((all_live >> lane) & 1) a.w.live[nxt][s_base[0] + bl + __popc(all_live & below)] = sl;
+        if (p_seed) a.w.seeds[nxt][s_base[1] + bs + __popc(ms & below)] = i;
     }
-    add_counters(a.counters, 0ull, 0ull, c_upd, 0ull, 0ull);
+    add_counters(a.counters, 0, 0, c_upd, 0, 0);
 }
 
-// ---- fused round: a4-a11 for every live candidate of round tau in one launch
-//
-// A block takes a slice of the round's live list whose ends are moved to seed boundaries (the
-// live candidates of a seed are contiguous in the list, at most kGroup of them), so each seed is
-// handled by exactly one block.  Three phases, each with its own mapping of threads to work:
-//   phase 1  one thread per candidate of the slice: propagation, window and chi2 (a4-a9); its
-//            prediction (or, when it does not cross its layer, its state) and its sorted hit
-//            children stay in shared memory;
-//   merge    eight lanes per seed: the N best children of the seed (a10) by 64-bit (score,
-//            parent slot) keys reduced with warp shuffles; every child becomes a descriptor in
-//            shared memory, and the seed's next-round list entries are reserved in one go (its
-//            candidates stay contiguous there);
-//   update   one thread per child descriptor: the Joseph update from the parent's prediction in
-//            shared memory (a11), the child's state, meta and trail.
-// Against two kernels per round (a thread per candidate, then eight lanes per seed for merge and
-// update) this keeps the prediction and child records (112 + 80 B per candidate) out of HBM, and
-// the update no longer idles the lanes of the seed's empty slots.  A child whose update fails
-// keeps its reserved list entry with a dead meta, which the next round skips.  The FP64 redo of a
-// flagged update (k_rescue) finds its parent's prediction in the prediction array, written for
-// flagged children only.
-
-template <class F> constexpr int rec_vecs() { return (int)(state_bytes<F>() / 16); }
-constexpr int kChildVecs(bool mod) { return mod ? 3 : 2; }   // int4 words of a child descriptor
-// Shared memory of k_round for a block of th threads: records [rec_vecs][th] of 16-byte vectors,
-// hit children chi2 / binned index / hit id [kGroup][th] each, per item a header and its slot
-// meta (int4 each) and its slot, the first item of each seed (th + 1), and 4 th child
-// descriptors (a merge chunk of th / 2 seeds has at most 4 th children).
-template <class F, bool MOD> constexpr size_t round_smem_bytes(int th) {
-    return (size_t)th * (16 * rec_vecs<F>() + 12 * kGroup + 16 + 16 + 8) + 16 + (size_t)4 * th * 16 * kChildVecs(MOD);
-}
-
-template <class F, int TH, int MINB, bool BWD = false, bool MOD = false>
-__global__ void __launch_bounds__(TH, MINB) k_round(BuildArgs a, int tau) {
-    static_assert(TH % 32 == 0 && TH >= 64, "whole warps, at least two per block");
-    __shared__ DevGeom g;
-    __shared__ int s_be[2];
-    __shared__ int s_wsum[TH / 32];
-    __shared__ int s_nchild;
-    extern __shared__ __align__(16) unsigned char dsm[];
-    using V = typename Vec16<F>::T;
-    constexpr int RV = rec_vecs<F>();                       // 16-byte vectors of a state record
-    constexpr int PV = (int)(pred_bytes<F>() / 16);         // ... of a prediction record
-    constexpr int per = 16 / (int)sizeof(F);
-    constexpr int CV = kChildVecs(MOD);
-    constexpr int kChunkSeeds = TH / 2;                     // seeds merged before their updates
-    V* s_rec = reinterpret_cast<V*>(dsm);                   // [RV][TH]
-    float* s_x2 = reinterpret_cast<float*>(dsm + (size_t)16 * RV * TH);   // [kGroup][TH]
-    int* s_hq = reinterpret_cast<int*>(s_x2 + kGroup * TH);
-    int* s_id = s_hq + kGroup * TH;
-    int4* s_hdr = reinterpret_cast<int4*>(s_id + kGroup * TH);   // (n hits, non-hit kind, its score, b2)
-    int4* s_imeta = s_hdr + TH;                                  // the item's slot meta
-    int4* s_child = s_imeta + TH;                                // [4 TH][CV] child descriptors
-    int* s_slot = reinterpret_cast<int*>(s_child + 4 * TH * CV);
-    int* s_first = s_slot + TH;                                  // TH + 1
-    load_geom_smem(a.geom, g);
-    const DevParams& P = a.P;
-    const int tx = threadIdx.x, lane = tx & 31, wid = tx >> 5;
-    const int cur = tau & 1, nxt = cur ^ 1;
-    const int n = a.w.rcounts[tau];
-    const int* __restrict__ list = a.w.live[cur];
-    int* cnt_live = a.w.rcounts + tau + 1;
-    int* cnt_resc = a.w.rcounts + kRescueCountBase + tau;
-    constexpr int kSpan = TH - (kGroup - 1);   // nominal slice: at most TH items once its ends move
-    const int ntiles = (n + kSpan - 1) / kSpan;
-    unsigned long long c_steps = 0, c_chi2 = 0, c_tested = 0, c_newton = 0, c_upd = 0;
-    for (int tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-        if (wid == 0) {
-            // lanes 0-7: the eight positions from the nominal start, lanes 8-15: from the nominal
-            // end; one of each eight starts a seed (or lies past the list)
-            const int p = (tile + (lane >> 3)) * kSpan + (lane & 7);
-            bool first = false;
-            if (lane < 16) first = p >= n || p == 0 || (__ldg(list + p) >> 3) != (__ldg(list + p - 1) >> 3);
-            const unsigned m = __ballot_sync(kFull, first);
-            if (lane == 0) {
-                s_be[0] = min(n, tile * kSpan + __ffs(m & 0xffu) - 1);
-                s_be[1] = min(n, (tile + 1) * kSpan + __ffs((m >> 8) & 0xffu) - 1);
-            }
-        }
-        __syncthreads();
-        const int items = s_be[1] - s_be[0];
-
-        // ---- phase 1: a4-a9 for the slice's candidates, one per thread
-        const int sl = tx < items ? __ldg(list + s_be[0] + tx) : -1;
-        s_slot[tx] = sl;
-        if (sl >= 0) {
-            const int4 si = __ldg(a.w.sinfo + sl / kGroup);
-            const int4 mt = a.w.meta[cur][sl];
-            s_imeta[tx] = mt;
-            int nh_kind = K_NONE, n_h = 0, b2 = -1;
-            float nh_score = 0.0f;
-            if (mt.w != 0) {   // (0: dropped after the selection, its FP64 update redo failed)
-                StateT<F> t;
-                load_state_rec(a.w.st[cur] + (int64_t)sl * state_bytes<F>(), t);
-                const DevLayer& L = g.layers[g.plan[si.x + tau]];
-                const float score = __int_as_float(mt.x);
-                const int nholes = (mt.z >> 8) & 0xff;
-                PredT<F> q;
-                F dir[4];
-                int newton = 0;
-                const int r = propagate_core<F, F, BWD>(L, g.cB, P.material, t, t.c, q, q.c, newton, dir);
-                c_newton += newton;
-                int b1m = -1, b2id = 0, b1id = 0, b1q = -1;
-                float b1x = 0.0f, b2x = 0.0f;
-                if (r == 0) {   // not crossed: the child is the unchanged state
-                    nh_kind = K_SKIP;
-                    nh_score = score;
-                    F f[kStateWords];
-                    f[0] = t.xh; f[1] = t.yh; f[2] = t.zh; f[3] = t.xl; f[4] = t.yl; f[5] = t.zl;
-                    f[6] = t.k; f[7] = t.phi; f[8] = t.th;
-#pragma unroll
-                    for (int q2 = 0; q2 < 21; ++q2) f[9 + q2] = t.c[q2];
-                    f[30] = t.tl; f[31] = t.pl;
-#pragma unroll
-                    for (int v = 0; v < RV; ++v) s_rec[v * TH + tx] = pack16(f + per * v);
-                } else if (r > 0) {
-                    ++c_steps;
-                    if (nholes < P.max_holes) {
-                        nh_kind = K_MISS;
-                        nh_score = score - P.score_hole;
-                    } else {
-                        nh_kind = K_STOP;
-                        nh_score = score;
-                    }
-                    const FrameT<F> fr = frame_of(L.kind, q.xh, q.yh, dir[0], dir[1], dir[2], dir[3]);
-                    const WindowT<F> w = window(L, P, q, fr);
-                    const float eps = 1e-5f;
-                    const float fe0 = (w.eta - w.deta - eps - L.eta_lo) * L.eta_scale;
-                    const float fe1 = (w.eta + w.deta + eps - L.eta_lo) * L.eta_scale;
-                    const int e0 = fe0 >= 0.0f ? (int)fminf(floorf(fe0), (float)(L.n_eta - 1)) : 0;
-                    const int e1 = fe1 >= 0.0f ? (int)fminf(floorf(fe1), (float)(L.n_eta - 1)) : 0;
-                    const float pscale = L.n_phi * (1.0f / kTwoPi);
-                    const int f0 = (int)floorf((w.phi - w.dphi - eps + kPi) * pscale);
-                    const int f1 = (int)floorf((w.phi + w.dphi + eps + kPi) * pscale);
-                    int nf = f1 - f0 + 1;
-                    int fa = f0 % L.n_phi;
-                    if (fa < 0) fa += L.n_phi;
-                    if (nf >= L.n_phi) {
-                        nf = L.n_phi;
-                        fa = 0;
-                    }
-                    const int run1 = min(nf, L.n_phi - fa), run2 = nf - run1;
-                    const int64_t bb = (int64_t)si.w * g.bins_per_event + L.bin_base;
-                    for (int ie = e0; ie <= e1; ++ie) {
-                        const int64_t rowb = bb + (int64_t)ie * L.n_phi;
-                        for (int run = 0; run < 2; ++run) {
-                            const int b0 = run == 0 ? fa : 0;
-                            const int nb = run == 0 ? run1 : run2;
-                            if (nb <= 0) continue;
-                            const int q0 = __ldg(a.H.bin_start + rowb + b0);
-                            const int q1 = __ldg(a.H.bin_start + rowb + b0 + nb);
-                            for (int hq = q0; hq < q1; ++hq) {
-                                ++c_tested;
-                                const float2 ep = __ldg(a.H.hb_ep + hq);
-                                if (fabs(F(ep.x) - w.eta) <= w.deta && fabs(wrap_pi(F(ep.y) - w.phi)) <= w.dphi) {
-                                    ++c_chi2;
-                                    F m[3], v[6];
-                                    int id, md = -1;
-                                    F x2f;
-                                    bool okx;
-                                    if constexpr (MOD) {
-                                        load_hit(a.H.hb_pay, hq, m, v, &id, &md);
-                                        okx = md >= 0 ? module_chi2_dir(q, fr, dir, g.mods, md, g.cB, m, v, x2f)
-                                                      : chi2_hit(fr, q, m[0], m[1], m[2], v, x2f);
-                                    } else {
-                                        load_hit(a.H.hb_pay, hq, m, v, &id);
-                                        okx = chi2_hit(fr, q, m[0], m[1], m[2], v, x2f);
-                                    }
-                                    if (okx && x2f < F(P.chi2_cut)) {
-                                        const float x2 = float(x2f);   // scores and child order in FP32
-                                        if (MOD && md >= 0) {
-                                            if (b1m < 0 || x2 < b1x || (x2 == b1x && id < b1id)) {
-                                                if (b1m >= 0 && md != b1m) {   // the previous b1 becomes b2
-                                                    b2 = b1q; b2x = b1x; b2id = b1id;
-                                                }
-                                                b1q = hq; b1x = x2; b1id = id; b1m = md;
-                                            } else if (md != b1m && (b2 < 0 || x2 < b2x || (x2 == b2x && id < b2id))) {
-                                                b2 = hq; b2x = x2; b2id = id;
-                                            }
-                                        }
-                                        // insert into the sorted list (kept to its first kGroup entries)
-                                        int jj = n_h < kGroup ? n_h : kGroup - 1;
-                                        const bool fits = n_h < kGroup || x2 < s_x2[jj * TH + tx] ||
-                                                          (x2 == s_x2[jj * TH + tx] && id < s_id[jj * TH + tx]);
-                                        if (fits) {
-                                            while (jj > 0 && (x2 < s_x2[(jj - 1) * TH + tx] ||
-                                                              (x2 == s_x2[(jj - 1) * TH + tx] &&
-                                                               id < s_id[(jj - 1) * TH + tx]))) {
-                                                s_x2[jj * TH + tx] = s_x2[(jj - 1) * TH + tx];
-                                                s_id[jj * TH + tx] = s_id[(jj - 1) * TH + tx];
-                                                s_hq[jj * TH + tx] = s_hq[(jj - 1) * TH + tx];
-                                                --jj;
-                                            }
-                                            s_x2[jj * TH + tx] = x2;
-                                            s_id[jj * TH + tx] = id;
-                                            s_hq[jj * TH + tx] = hq;
-                                            if (n_h < kGroup) ++n_h;
-                                        }
-                                    }
-                                }
-                            }
-                        }
-                    }
-                    F f[kPredWords];
-                    f[0] = q.xh; f[1] = q.yh; f[2] = q.zh; f[3] = q.xl; f[4] = q.yl; f[5] = q.zl;
-                    f[6] = q.k; f[7] = q.phi; f[8] = q.th;
-#pragma unroll
-                    for (int q2 = 0; q2 < 15; ++q2) f[9 + q2] = q.c[q2];
-                    f[24] = q.tl; f[25] = q.pl; f[26] = F(0); f[27] = F(0);
-#pragma unroll
-                    for (int v = 0; v < PV; ++v) s_rec[v * TH + tx] = pack16(f + per * v);
-                }
-            }
-            s_hdr[tx] = make_int4(n_h, nh_kind, __float_as_int(nh_score), MOD ? b2 : -1);
-        }
-        __syncthreads();
-
-        // ---- the slice's seeds: the first item of each (block-wide count of seed starts)
-        int nseeds;
-        {
-            const bool first = sl >= 0 && (tx == 0 || (s_slot[tx - 1] >> 3) != (sl >> 3));
-            const unsigned m = __ballot_sync(kFull, first);
-            if (lane == 0) s_wsum[wid] = __popc(m);
-            __syncthreads();
-            int off = 0, tot = 0;
-#pragma unroll
-            for (int k = 0; k < TH / 32; ++k) {
-                const int v = s_wsum[k];
-                off += k < wid ? v : 0;
-                tot += v;
-            }
-            if (first) s_first[off + __popc(m & ((1u << lane) - 1u))] = tx;
-            if (tx == 0) s_first[tot] = items;
-            nseeds = tot;
-        }
-
-        const int slot = lane & 7, gbase = lane & ~7;
-        for (int sbase = 0; sbase < nseeds; sbase += kChunkSeeds) {
-            const int send = min(nseeds, sbase + kChunkSeeds);
-            if (tx == 0) s_nchild = 0;
-            __syncthreads();
-            // ---- merge: eight lanes per seed (lane = parent slot / child rank), a10
-            for (int wg = sbase + wid * 4; wg < send; wg += TH / kGroup) {   // uniform over the warp
-                const int gi = wg + (lane >> 3);
-                const bool gact = gi < send;
-                const int j0 = gact ? s_first[gi] : 0, j1 = gact ? s_first[gi + 1] : 0;
-                const int i = gact ? (s_slot[j0] >> 3) : 0;
-                const int4 si = gact ? __ldg(a.w.sinfo + i) : make_int4(0, 0, 0, 0);
-                int jr = -1;   // this slot's item in the slice (live candidates only)
-                for (int jj = j0; jj < j1; ++jj)
-                    if ((s_slot[jj] & 7) == slot) jr = jj;
-                const int4 mt = !gact ? make_int4(0, 0, 0, 0) : jr >= 0 ? s_imeta[jr] : a.w.meta[cur][i * kGroup + slot];
-                const float score = __int_as_float(mt.x);
-                const bool alive = mt.w != 0;
-                const bool stopped = ((mt.z >> 16) & 1) != 0;
-
-                int nh_kind = K_NONE;
-                float nh_score = -kBig;
-                int b1q = -1, b2q = -1;
-                float lx[kGroup];
-                int lq[kGroup];
-#pragma unroll
-                for (int jj = 0; jj < kGroup; ++jj) {
-                    lx[jj] = kBig;
-                    lq[jj] = 0;
-                }
-                if (alive) {
-                    if (stopped) {
-                        nh_kind = K_CARRY;
-                        nh_score = score;
-                    } else if (jr >= 0) {
-                        const int4 h = s_hdr[jr];
-                        nh_kind = h.y;
-                        nh_score = __int_as_float(h.z);
-#pragma unroll
-                        for (int jj = 0; jj < kGroup; ++jj)
-                            if (jj < h.x) {
-                                lx[jj] = s_x2[jj * TH + jr];
-                                lq[jj] = s_hq[jj * TH + jr];
-                            }
-                        if constexpr (MOD) {
-                            b2q = h.w;
-                            b1q = h.x > 0 ? lq[0] : -1;
-                        }
-                    }
-                }
-                const float ovl_bonus = MOD && b2q >= 0 ? P.score_overlap : 0.0f;
-
-                bool nh_avail = nh_kind != K_NONE;
-                int my_parent = -1, my_kind = K_NONE, my_q = 0, my_b1 = -1, my_b2 = -1;
-                float my_x2 = 0.0f, my_score = 0.0f;
-                for (int r = 0; r < P.max_cands; ++r) {
-                    const bool has_hit = lx[0] < kBig;
-                    float hit_score = score + P.score_hit - lx[0];
-                    if constexpr (MOD) hit_score += ovl_bonus;
-                    int hk = K_NONE;
-                    float hs = 0.0f;
-                    if (has_hit && (!nh_avail || hit_score >= nh_score)) {
-                        hk = K_HIT;
-                        hs = hit_score;
-                    } else if (nh_avail) {
-                        hk = nh_kind;
-                        hs = nh_score;
-                    }
-                    unsigned long long best = hk != K_NONE ? order_key(hs, slot) : 0ull;
-#pragma unroll
-                    for (int off = 1; off < kGroup; off <<= 1) {
-                        const unsigned long long o = __shfl_xor_sync(kFull, best, off);
-                        best = o > best ? o : best;
-                    }
-                    const bool valid = best != 0ull;
-                    const int wslot = kGroup - 1 - (int)(best & 7ull);
-                    const int src = gbase + wslot;
-                    const int w_kind = shfl_i(hk, src);
-                    const int w_q = shfl_i(lq[0], src);
-                    const float w_x2 = shfl_f(lx[0], src);
-                    const float w_score = shfl_f(hs, src);
-                    if (valid && slot == r) {
-                        my_parent = wslot;
-                        my_kind = w_kind;
-                        my_q = w_q;
-                        my_x2 = w_x2;
-                        my_score = w_score;
-                    }
-                    if constexpr (MOD) {
-                        const int w_b1 = shfl_i(b1q, src), w_b2 = shfl_i(b2q, src);
-                        if (valid && slot == r) {
-                            my_b1 = w_b1;
-                            my_b2 = w_b2;
-                        }
-                    }
-                    if (valid && slot == wslot) {
-                        if (hk == K_HIT) {
-#pragma unroll
-                            for (int jj = 0; jj < kGroup - 1; ++jj) {
-                                lx[jj] = lx[jj + 1];
-                                lq[jj] = lq[jj + 1];
-                            }
-                            lx[kGroup - 1] = kBig;
-                        } else {
-                            nh_avail = false;
-                        }
-                    }
-                }
-
-                // the child of rank `slot`: its parent's meta and record, descriptor and list entry
-                const int psrc = gbase + (my_parent >= 0 ? my_parent : slot);
-                const int4 pm = make_int4(shfl_i(mt.x, psrc), shfl_i(mt.y, psrc), shfl_i(mt.z, psrc), shfl_i(mt.w, psrc));
-                const int pj = shfl_i(jr, psrc);
-                const int csl = i * kGroup + slot;
-                const bool has_child = gact && my_kind != K_NONE;
-                const bool more = gact && tau + 1 < si.z;
-                // live next round unless stopped (its parent's stop carried, or a stop here) or its
-                // update fails (its entry then meets a dead meta)
-                const bool pot_live = has_child && more && my_kind != K_STOP && my_kind != K_CARRY &&
-                                      ((pm.z >> 16) & 1) == 0;
-                const unsigned mc = __ballot_sync(kFull, has_child), ml = __ballot_sync(kFull, pot_live);
-                int bc = 0, bl = 0;
-                if (lane == 0) {
-                    if (mc) bc = atomicAdd(&s_nchild, __popc(mc));
-                    if (ml) bl = atomicAdd(cnt_live, __popc(ml));
-                }
-                bc = __shfl_sync(kFull, bc, 0);
-                bl = __shfl_sync(kFull, bl, 0);
-                const unsigned below = (1u << lane) - 1u;
-                if (pot_live) a.w.live[nxt][bl + __popc(ml & below)] = csl;
-                if (has_child) {
-                    const int c = bc + __popc(mc & below);
-                    int4* d = s_child + c * CV;
-                    d[0] = make_int4(csl, my_kind | (my_parent << 4) | ((pj + 1) << 8), my_q, __float_as_int(my_x2));
-                    d[1] = make_int4(__float_as_int(my_score), pm.y, pm.z, g.plan[si.x + tau]);
-                    if constexpr (MOD) d[2] = make_int4(my_b1, my_b2, 0, 0);
-                } else if (gact) {
-                    a.w.meta[nxt][csl] = make_int4(0, 0, 0, 0);
-                }
-                // no live child left (plan ended, every child stopped or none): the seed ends here
-                const bool any_live = ((ml >> gbase) & 0xffu) != 0u;
-                if (gact && slot == 0 && !any_live) a.w.fin[i] = nxt | ((tau + 1) << 1);
-            }
-            __syncthreads();
-
-            // ---- update: one thread per child (a11)
-            const int nc = s_nchild;
-            for (int c0 = 0; c0 < nc; c0 += TH) {   // uniform over the block
-                const int c = c0 + tx;
-                const bool act = c < nc;
-                int4 d0 = make_int4(0, 0, 0, 0), d1 = make_int4(0, 0, 0, 0);
-                int my_b1 = -1, my_b2 = -1;
-                if (act) {
-                    d0 = s_child[c * CV];
-                    d1 = s_child[c * CV + 1];
-                    if constexpr (MOD) {
-                        const int4 d2 = s_child[c * CV + 2];
-                        my_b1 = d2.x;
-                        my_b2 = d2.y;
-                    }
-                }
-                const int csl = d0.x, my_kind = d0.y & 15, my_parent = (d0.y >> 4) & 15, pj = (d0.y >> 8) - 1;
-                const int my_q = d0.z;
-                const float my_x2 = __int_as_float(d0.w), my_score = __int_as_float(d1.x);
-                const int i = csl / kGroup, cslot = csl % kGroup;
-                bool c_alive = act, c_stopped = ((d1.z >> 16) & 1) != 0;
-                float chi2s = __int_as_float(d1.y);
-                int nfound = d1.z & 0xff, nholes = (d1.z >> 8) & 0xff;
-                int code = MKGB_HIT_STOP;
-                bool rescue = false;
-                int ovl = -1;
-                if (act) {
-                    const int psl = i * kGroup + my_parent;
-                    unsigned char* dst = a.w.st[nxt] + (int64_t)csl * state_bytes<F>();
-                    if (my_kind == K_CARRY) {
-                        copy_state_rec<F>(a.w.st[cur] + (int64_t)psl * state_bytes<F>(), dst);
-                    } else if (my_kind == K_SKIP) {
-                        V* d4 = reinterpret_cast<V*>(dst);
-#pragma unroll
-                        for (int v = 0; v < RV; ++v) d4[v] = s_rec[v * TH + pj];
-                        code = MKGB_HIT_SKIP;
-                    } else {
-                        const DevLayer& L = g.layers[d1.w];
-                        PredT<F> pq;
-                        {
-                            F f[kPredWords];
-#pragma unroll
-                            for (int v = 0; v < PV; ++v) unpack16(s_rec[v * TH + pj], f + per * v);
-                            pq.xh = f[0]; pq.yh = f[1]; pq.zh = f[2]; pq.xl = f[3]; pq.yl = f[4]; pq.zl = f[5];
-                            pq.k = f[6]; pq.phi = f[7]; pq.th = f[8];
-#pragma unroll
-                            for (int q2 = 0; q2 < 15; ++q2) pq.c[q2] = f[9 + q2];
-                            pq.tl = f[24];
-                            pq.pl = f[25];
-                        }
-                        StateT<F> t;
-                        if (my_kind == K_HIT) {
-                            F m[3], v[6];
-                            int id, md = -1;
-                            if constexpr (MOD)
-                                load_hit(a.H.hb_pay, my_q, m, v, &id, &md);
-                            else
-                                load_hit(a.H.hb_pay, my_q, m, v, &id);
-                            float kap = 0.0f;
-                            bool ok;
-                            if (MOD && md >= 0) {   // a module hit: the update on its module's plane (Sec. 3.1)
-                                F x2u;
-                                ok = module_update(L.kind, pq, g.mods, md, g.cB, m, v, 0.0f, t, x2u, kap) == 0;
-                                if (my_b2 >= 0) {   // the overlap hit: b1 unless the hit is on b1's module
-                                    const int m1 = __float_as_int(__ldg(a.H.hb_pay + 3 * (int64_t)my_b1 + 2).z);
-                                    const int oq = md != m1 ? my_b1 : my_b2;
-                                    ovl = __float_as_int(__ldg(a.H.hb_pay + 3 * (int64_t)oq).w);
-                                }
-                            } else {
-                                ok = kalman_update(L.kind, pq, m[0], m[1], m[2], v, t, &kap);
-                            }
-                            if (ok) {
-                                chi2s += my_x2;
-                                ++nfound;
-                                ++c_upd;
-                                code = id;
-                                // FP32 cannot resolve an innovation covariance this ill-conditioned:
-                                // k_rescue redoes the update in FP64 from the parent's prediction
-                                rescue = sizeof(F) == 4 && P.kappa_fp64 > 0.0f && kap > P.kappa_fp64;
-                                if (rescue) store_pred_rec(a.w.pr + (int64_t)psl * pred_bytes<F>(), pq);
-                            } else {
-                                c_alive = false;
-                            }
-                        } else {
-                            pred_to_state(L.kind, pq, t);
-                            if (my_kind == K_MISS) {
-                                ++nholes;
-                                code = MKGB_HIT_MISS;
-                            } else {   // K_STOP
-                                c_stopped = true;
-                            }
-                        }
-                        store_state_rec(dst, t);
-                    }
-                    a.w.trail[((int64_t)i * a.max_steps + tau) * kGroup + cslot] = ((code + 4) << 3) | my_parent;
-                    if (MOD && a.w.otrail)
-                        a.w.otrail[((int64_t)i * a.max_steps + tau) * kGroup + cslot] = c_alive ? ovl : -1;
-                    a.w.meta[nxt][csl] = pack_meta(my_score, chi2s, nfound, nholes, c_stopped, c_alive);
-                }
-                const unsigned m0 = __ballot_sync(kFull, rescue);
-                int b0 = 0;
-                if (lane == 0 && m0) b0 = atomicAdd(cnt_resc, __popc(m0));
-                b0 = __shfl_sync(kFull, b0, 0);
-                if (rescue) a.w.rescue[b0 + __popc(m0 & ((1u << lane) - 1u))] = csl;
-            }
-            __syncthreads();   // the next chunk's merge reuses the descriptors
-        }
-    }
-    add_counters(a.counters, c_steps, c_chi2, c_upd, c_tested, c_newton);
-}
-
-// ---- FP64 redo of the round's flagged updates (kept children of round tau whose innovation
-// covariance had a condition estimate above kappa_fp64); one thread per child
-__global__ void __launch_bounds__(kThreads) k_rescue(BuildArgs a, int tau) {
-    __shared__ DevGeom g;
-    load_geom_smem(a.geom, g);
-    const int nxt = (tau & 1) ^ 1;
-    const int n = a.fused ? a.w.rcounts[kRescueCountBase + tau] : a.w.counts[4];
-    for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < n; r += gridDim.x * blockDim.x) {
-        const int csl = a.w.rescue[r];
-        const int i = csl / kGroup;
-        const int slot = csl % kGroup;
-        const int v = a.w.trail[((int64_t)i * a.max_steps + tau) * kGroup + slot];
-        const int psl = i * kGroup + (v & 7);
-        const int4 si = a.w.sinfo[i];
-        const int lkind = g.layers[g.plan[si.x + tau]].kind;
-        Pred pq;
-        load_pred_rec(a.w.pr + (int64_t)psl * pred_bytes<float>(), pq);
-        PredT<double> qd;
-        qd.xh = pq.xh; qd.yh = pq.yh; qd.zh = pq.zh; qd.xl = pq.xl; qd.yl = pq.yl; qd.zl = pq.zl;
-        qd.k = pq.k; qd.phi = pq.phi; qd.th = pq.th; qd.tl = pq.tl; qd.pl = pq.pl;
-#pragma unroll
-        for (int q = 0; q < 15; ++q) qd.c[q] = pq.c[q];
-        // the hit: its binned index is not in the trail (which holds the hit id), so it is looked
-        // up through the hit id in the payload's original order
-        const int id = (v >> 3) - 4;
-        double m[3], vv[6];
-        int md;
-        load_hit(a.H.pay, id, m, vv, nullptr, &md);
-        StateT<double> td;
-        bool ok;
-        if (md >= 0) {
-            double x2u;
-            float kap;
-            ok = module_update(lkind, qd, g.mods, md, g.cB, m, vv, 0.0f, td, x2u, kap) == 0;
-        } else {
-            ok = kalman_update(lkind, qd, m[0], m[1], m[2], vv, td);
-        }
-        if (ok) {
-            State t;
-            narrow_state(td, t);
-            store_state_rec(a.w.st[nxt] + (int64_t)csl * state_bytes<float>(), t);
-        } else {
-            a.w.meta[nxt][csl].w = 0;   // dropped; k_find skips it
-        }
-    }
-}
-
-// ---- best candidate per seed and its hit list (a13); 8 lanes per seed
-template <class F>
+// ---- best candidate per seed and its hit list (a13); one thread per seed.  REDO: the seeds that the
+// first launch left because the last update of their best candidate is one for FP64.
+template <class F, bool REDO>
 __global__ void __launch_bounds__(kThreads) k_finish(BuildArgs a) {
-    const int lane = threadIdx.x & 31, slot = lane & 7, gbase = lane & ~7;
-    const int gi = (blockIdx.x * blockDim.x + threadIdx.x) >> 3;
-    const bool gact = gi < a.S.n;
-    const int i = gact ? gi : 0;
-    const int finv = gact ? a.w.fin[i] : -1;
-    const int fin = finv >= 0 ? finv & 1 : -1, rounds = finv >= 0 ? finv >> 1 : 0;
-    int4 mt = make_int4(0, 0, 0, 0);
-    if (fin >= 0) mt = a.w.meta[fin][i * kGroup + slot];
-    const unsigned am = __ballot_sync(kFull, mt.w != 0);
-    const unsigned gm = (am >> gbase) & 0xffu;
-    if (!gact) return;
-    const int best = gm ? __ffs(gm) - 1 : -1;
+    if (!REDO) next_kernel_may_start();
+    wait_for_last_kernel();
+    int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= (REDO ? a.w.counts[4] : a.S.n)) return;
+    if (REDO) i = a.w.redo[i];
+    const int rounds = a.w.fin[i];   // rounds searched, -1 none
     const int seed = a.S.order[i];
+    int4 mt = make_int4(0, 0, 0, 0);
+    int best = -1;
+    StateT<F> t;
+    // the last round's children still have to take their hits: the best one, the next if that fails
+    for (int r = 0; rounds > 0 && best < 0 && r < kGroup; ++r) {
+        const int cs = i * kGroup + r;
+        mt = a.w.meta[rounds & 1][slot_at(cs)];
+        if (mt.w == 0) continue;
+        F f[kStateWords];
+        F m[3] = {F(0), F(0), F(0)}, v[6] = {F(0), F(0), F(0), F(0), F(0), F(0)};
+        int4 d = pack_child(0, K_MISS, (mt.z >> 17) & 1, 0, 0.0f, 0);   // stopped: its record is a prediction
+        if ((mt.z >> 16) & 1) {
+            load_rec<F, kStateWords>(a.w.stop, i * kGroup + ((mt.z >> 18) & 7), f);
+        } else {
+            d = a.w.child[slot_at(cs)];
+            load_rec<F, kStateWords>(a.w.rec[(rounds & 1) ^ 1], i * kGroup + child_parent(d), f);
+            if (child_kind(d) == K_HIT) load_hit(a.H.hb_pay, d.y, m, v, nullptr);
+        }
+        int fail = child_state(a, d, f, m, v, t);
+        if (fail == 2) {
+            if constexpr (REDO) {
+                Pred q;
+                unpack_pred(f, q);
+                fail = update_fp64(child_surface(d), q, a.H.hb_pay, d.y, t) ? 0 : 1;
+            } else {
+                a.w.redo[atomicAdd(a.w.counts + 4, 1)] = i;
+                return;
+            }
+        }
+        if (fail == 0) best = r;
+    }
     int* hrow = a.out.hits + (int64_t)seed * a.out.max_plan;
     int* orow = a.out.ovl ? a.out.ovl + (int64_t)seed * a.out.max_plan : nullptr;
-    for (int q = slot; q < a.out.max_plan; q += kGroup) {
-        hrow[q] = MKGB_HIT_PRE;
-        if (orow) orow[q] = -1;
-    }
-    __syncwarp(0xffu << gbase);
-    if (slot != (best >= 0 ? best : 0)) return;
     float* po = a.out.params + 6 * (int64_t)seed;
     float* co = a.out.cov + 21 * (int64_t)seed;
+    int q0 = a.out.max_plan, q1 = a.out.max_plan;   // steps of the row that the search covered
     if (best >= 0) {
-        StateT<F> t;
-        load_state_rec(a.w.st[fin] + (int64_t)(i * kGroup + best) * state_bytes<F>(), t);
         store_state6(t, po, co);
         a.out.chi2[seed] = __int_as_float(mt.y);
         a.out.score[seed] = __int_as_float(mt.x);
         a.out.nfound[seed] = mt.z & 0xff;
         a.out.nholes[seed] = (mt.z >> 8) & 0xff;
         const int4 si = a.w.sinfo[i];
-        // a seed whose candidates had all stopped before its plan ended (fused rounds finish it
-        // then): its later plan steps are those of a stopped candidate
-        for (int tau = rounds; tau < si.z; ++tau) {
-            hrow[si.y + tau] = MKGB_HIT_STOP;
-            if (orow) orow[si.y + tau] = -1;
-        }
+        q0 = si.y;
+        q1 = si.y + min(rounds, si.z);
         int s_ = best;
         for (int tau = min(rounds, si.z) - 1; tau >= 0; --tau) {
-            const int64_t at = ((int64_t)i * a.max_steps + tau) * kGroup + s_;
+            const int64_t at = (int64_t)tau * a.slots + slot_at(i * kGroup + s_);
             const int v = a.w.trail[at];
-            hrow[si.y + tau] = (v >> 3) - 4;
-            if (orow && a.w.otrail) orow[si.y + tau] = a.w.otrail[at];
+            const int code = (v >> 3) - 4;   // a hit: its binned index
+            hrow[si.y + tau] = code >= 0 ? __float_as_int(__ldg(a.H.hb_pay + 3 * (int64_t)code).w) : code;
             s_ = v & 7;
         }
     } else {
@@ -1260,6 +758,11 @@ __global__ void __launch_bounds__(kThreads) k_finish(BuildArgs a) {
         a.out.score[seed] = -INFINITY;
         a.out.nfound[seed] = 0;
         a.out.nholes[seed] = 0;
+    }
+    for (int q = 0; q < a.out.max_plan; ++q) {
+        const bool covered = q >= q0 && q < q1;
+        if (!covered) hrow[q] = MKGB_HIT_PRE;
+        if (orow) orow[q] = -1;   // no module hits, no overlap hits
     }
 }
 
@@ -1276,32 +779,33 @@ namespace {
 
 // Carves the work buffers out of one allocation (256-byte aligned pieces); with base == nullptr
 // only the total size is computed.
-size_t layout_build_work(char* base, int n_seeds, int max_plan_len, int word_bytes, bool with_ovl, BuildWork* w) {
-    const size_t ns = (size_t)n_seeds, slots = ns * kGroup, wb = (size_t)word_bytes;
+size_t layout_build_work(char* base, int n_seeds, int max_plan_len, int word_bytes, BuildWork* w) {
+    const size_t ns = (size_t)n_seeds, slots = tile_slots(n_seeds), wb = (size_t)word_bytes;
     size_t off = 0;
     auto take = [&](size_t bytes) {
         char* r = base ? base + off : nullptr;
         off += (bytes + 255) & ~(size_t)255;
         return r;
     };
-    BuildWork t;
-    t.st[0] = reinterpret_cast<unsigned char*>(take(slots * kStateWords * wb));
-    t.st[1] = reinterpret_cast<unsigned char*>(take(slots * kStateWords * wb));
+    BuildWork t = {};
+    t.rec[0] = reinterpret_cast<unsigned char*>(take(slots * kStateWords * wb));
+    t.rec[1] = reinterpret_cast<unsigned char*>(take(slots * kStateWords * wb));
+    t.stop = reinterpret_cast<unsigned char*>(take(slots * kStateWords * wb));
     t.meta[0] = reinterpret_cast<int4*>(take(slots * 16));
     t.meta[1] = reinterpret_cast<int4*>(take(slots * 16));
-    t.pr = reinterpret_cast<unsigned char*>(take(slots * kPredWords * wb));
-    t.ls = reinterpret_cast<int4*>(take(slots * 80));
+    t.child = reinterpret_cast<int4*>(take(slots * 16));
+    t.ls = reinterpret_cast<int4*>(take(slots * 32));
+    t.ls_more = reinterpret_cast<int4*>(take(slots * 48));
     t.live[0] = reinterpret_cast<int*>(take(slots * 4));
     t.live[1] = reinterpret_cast<int*>(take(slots * 4));
     t.seeds[0] = reinterpret_cast<int*>(take(ns * 4));
     t.seeds[1] = reinterpret_cast<int*>(take(ns * 4));
     t.sinfo = reinterpret_cast<int4*>(take(ns * 16));
     t.fin = reinterpret_cast<int*>(take(ns * 4));
-    t.trail = reinterpret_cast<int*>(take(ns * (size_t)max_plan_len * kGroup * 4));
-    t.otrail = with_ovl ? reinterpret_cast<int*>(take(ns * (size_t)max_plan_len * kGroup * 4)) : nullptr;
-    t.rescue = reinterpret_cast<int*>(take(slots * 4));
-    t.counts = reinterpret_cast<int*>(take(32 + 4 * kRoundCountInts));
-    t.rcounts = base ? t.counts + 8 : nullptr;
+    t.trail = reinterpret_cast<int*>(take(slots * (size_t)max_plan_len * 4));
+    t.redo = reinterpret_cast<int*>(take(slots * 4));
+    t.found = reinterpret_cast<int*>(take(slots * 4));
+    t.counts = reinterpret_cast<int*>(take(32));
     if (w) *w = t;
     return off;
 }
@@ -1340,142 +844,114 @@ __global__ void __launch_bounds__(kThreads) k_bw_seed(const DevGeom* __restrict_
 }
 
 // Launch shapes of the round kernels (threads per block, minimum resident blocks per SM), one of
-// which the autotuner picks: k_find x k_select.  The resident grid of each shape is computed once,
+// which the autotuner picks: k_move x k_find.  The resident grid of each shape is computed once,
 // before any capture.
-template <class F, int TH, int MINB, bool BWD = false, bool MOD = false> struct FindShape {
+template <class F, int TH, int MINB, bool BWD, bool REDO = false> struct MoveShape {
     static int grid(int n_sms) {
         static int g = 0;
-        if (!g) g = resident_grid((const void*)k_find<F, TH, MINB, BWD, MOD>, n_sms, TH);
+        if (!g) g = resident_grid((const void*)k_move<F, TH, MINB, BWD, REDO>, n_sms, TH);
         return g;
     }
     static void launch(cudaStream_t st, const BuildArgs& a, int tau, int n_sms) {
-        k_find<F, TH, MINB, BWD, MOD><<<grid(n_sms), TH, 0, st>>>(a, tau);
+        launch_next(k_move<F, TH, MINB, BWD, REDO>, REDO ? n_sms : grid(n_sms), TH, st, a, tau);
     }
 };
-template <class F, int TH, int MINB, bool MOD = false> struct SelectShape {
+template <class F, int TH, int MINB> struct FindShape {
     static int grid(int n_sms) {
         static int g = 0;
-        if (!g) g = resident_grid((const void*)k_select<F, TH, MINB, MOD>, n_sms, TH);
+        if (!g) g = resident_grid((const void*)k_find<F, TH, MINB>, n_sms, TH);
         return g;
     }
     static void launch(cudaStream_t st, const BuildArgs& a, int tau, int n_sms) {
-        k_select<F, TH, MINB, MOD><<<grid(n_sms), TH, 0, st>>>(a, tau);
+        launch_next(k_find<F, TH, MINB>, grid(n_sms), TH, st, a, tau);
+    }
+};
+template <class F, int TH, int MINB> struct MergeShape {
+    static int grid(int n_sms) {
+        static int g = 0;
+        if (!g) g = resident_grid((const void*)k_merge<F, TH, MINB>, n_sms, TH);
+        return g;
+    }
+    static void launch(cudaStream_t st, const BuildArgs& a, int tau, int n_sms) {
+        launch_next(k_merge<F, TH, MINB>, grid(n_sms), TH, st, a, tau);
     }
 };
 
-// The fused round kernel: dynamic shared memory set once per instantiation, resident grid.
-template <class F, int TH, int MINB, bool BWD = false, bool MOD = false> struct RoundShape {
-    static int grid(int n_sms) {
-        static int g = 0;
-        if (!g) {
-            const void* k = (const void*)k_round<F, TH, MINB, BWD, MOD>;
-            const size_t smem = round_smem_bytes<F, MOD>(TH);
-            cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-            int per_sm = 0;
-            if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, TH, smem) != cudaSuccess || per_sm < 1)
-                per_sm = 1;
-            g = n_sms * per_sm;
+// find_shape: k_move as blocks of 128 x 5, 128 x 4 (the default), 256 x 2, 64 x 8, 64 x 10, 128 x 3
+// (threads x resident blocks per SM): 128 registers a thread at 16 warps (no spills; 15.5 ms per
+// 64-event search), 96 at 20 (112 bytes spilled; 15.7), 138 at 12 (16.7; all with the former k_merge).  select_shape: k_find as
+// 128 x 6, 64 x 12 (80 registers), 128 x 8 (64 registers, 48 bytes spilled; 0.9 ms slower).
+template <class F, bool BWD, class Do> void with_move_shape(int shape, Do&& f) {
+    if constexpr (sizeof(F) == 8) {
+        f(MoveShape<F, 128, 1, BWD>());
+    } else if constexpr (BWD) {   // the backward search: one shape
+        f(MoveShape<F, 128, 4, BWD>());
+    } else {
+        switch (shape) {
+            case 0: f(MoveShape<F, 128, 5, BWD>()); break;
+            case 2: f(MoveShape<F, 256, 2, BWD>()); break;
+            case 3: f(MoveShape<F, 64, 8, BWD>()); break;
+            case 4: f(MoveShape<F, 64, 10, BWD>()); break;
+            case 5: f(MoveShape<F, 128, 3, BWD>()); break;
+            default: f(MoveShape<F, 128, 4, BWD>()); break;
         }
-        return g;
     }
-    static void launch(cudaStream_t st, const BuildArgs& a, int tau, int n_sms) {
-        k_round<F, TH, MINB, BWD, MOD><<<grid(n_sms), TH, round_smem_bytes<F, MOD>(TH), st>>>(a, tau);
-    }
-};
-
-template <class F, bool MOD> void prime_shapes_of(int n_sms) {
-    RoundShape<F, 128, 4, false, MOD>::grid(n_sms);
-    RoundShape<F, 128, 3, false, MOD>::grid(n_sms);
-    RoundShape<F, 256, 2, false, MOD>::grid(n_sms);
-    FindShape<F, 64, 8, false, MOD>::grid(n_sms);
-    FindShape<F, 128, 1, false, MOD>::grid(n_sms);
-    FindShape<F, 256, 1, false, MOD>::grid(n_sms);
-    SelectShape<F, 64, 10, MOD>::grid(n_sms);
-    SelectShape<F, 128, 5, MOD>::grid(n_sms);
-    SelectShape<F, 256, 2, MOD>::grid(n_sms);
 }
-
-template <class F> void prime_shapes(int n_sms) {
-    if (sizeof(F) == 4) {
-        FindShape<float, 128, 1, true>::grid(n_sms);
-        FindShape<float, 128, 1, true, true>::grid(n_sms);
-        RoundShape<float, 128, 4, true>::grid(n_sms);
-        RoundShape<float, 128, 4, true, true>::grid(n_sms);
-    }
-    prime_shapes_of<F, false>(n_sms);
-    prime_shapes_of<F, true>(n_sms);
-}
-
-template <class F, bool BWD = false, bool MOD = false>
-void launch_find(int shape, cudaStream_t st, const BuildArgs& a, int tau, int n_sms) {
-    if constexpr (BWD) {   // the backward search: one shape, FP32 only
-        FindShape<F, 128, 1, true, MOD>::launch(st, a, tau, n_sms);
-        return;
-    }
-    switch (shape) {
-        case 1: FindShape<F, 64, 8, false, MOD>::launch(st, a, tau, n_sms); break;
-        case 2: FindShape<F, 256, 1, false, MOD>::launch(st, a, tau, n_sms); break;
-        default: FindShape<F, 128, 1, false, MOD>::launch(st, a, tau, n_sms); break;
+template <class F, class Do> void with_find_shape(int shape, Do&& f) {
+    if constexpr (sizeof(F) == 8) {
+        f(FindShape<F, 128, 2>());
+    } else {
+        switch (shape) {
+            case 1: f(FindShape<F, 64, 12>()); break;
+            case 2: f(FindShape<F, 128, 8>()); break;
+            default: f(FindShape<F, 128, 6>()); break;
+        }
     }
 }
 
-// Fused round shapes: find_shape 3, 4, 5 = blocks of 128 x 4, 128 x 3, 256 x 2 (threads x resident
-// blocks per SM); the backward search takes 128 x 4.
-template <class F, bool BWD = false, bool MOD = false>
-void launch_round(int shape, cudaStream_t st, const BuildArgs& a, int tau, int n_sms) {
-    if constexpr (BWD) {
-        RoundShape<F, 128, 4, true, MOD>::launch(st, a, tau, n_sms);
-        return;
-    }
-    switch (shape) {
-        case 4: RoundShape<F, 128, 3, false, MOD>::launch(st, a, tau, n_sms); break;
-        case 5: RoundShape<F, 256, 2, false, MOD>::launch(st, a, tau, n_sms); break;
-        default: RoundShape<F, 128, 4, false, MOD>::launch(st, a, tau, n_sms); break;
-    }
-}
-
-template <class F, bool MOD = false>
-void launch_select(int shape, cudaStream_t st, const BuildArgs& a, int tau, int n_sms) {
-    switch (shape) {
-        case 1: SelectShape<F, 64, 10, MOD>::launch(st, a, tau, n_sms); break;
-        case 2: SelectShape<F, 256, 2, MOD>::launch(st, a, tau, n_sms); break;
-        default: SelectShape<F, 128, 5, MOD>::launch(st, a, tau, n_sms); break;
-    }
-}
-
-template <class F, bool BWD = false, bool MOD = false>
+template <class F, bool BWD = false>
 cudaError_t launch_rounds(cudaStream_t st, const BuildArgs& a, int n, int max_plan_len, int n_sms, int find_shape,
                           int select_shape) {
-    cudaError_t e = cudaMemsetAsync(a.w.counts, 0, 32 + 4 * kRoundCountInts, st);
+    cudaError_t e = cudaMemsetAsync(a.w.counts, 0, 32, st);
     if (e != cudaSuccess) return e;
     const int nb = (n + kThreads - 1) / kThreads;
-    k_start<F><<<nb, kThreads, 0, st>>>(a);
+    k_start<<<nb, kThreads, 0, st>>>(a);
     for (int tau = 0; tau < max_plan_len; ++tau) {
-        if (a.fused) {
-            launch_round<F, BWD, MOD>(find_shape, st, a, tau, n_sms);
-        } else {
-            launch_find<F, BWD, MOD>(find_shape, st, a, tau, n_sms);
-            launch_select<F, MOD>(select_shape, st, a, tau, n_sms);
+        with_move_shape<F, BWD>(find_shape, [&](auto s) { decltype(s)::launch(st, a, tau, n_sms); });
+        if constexpr (sizeof(F) == 4) {
+            if (a.P.kappa_fp64 > 0.0f && tau > 0) MoveShape<F, 64, 1, BWD, true>::launch(st, a, tau, n_sms);
         }
-        if (sizeof(F) == 4 && a.P.kappa_fp64 > 0.0f) k_rescue<<<n_sms, kThreads, 0, st>>>(a, tau);
+        with_find_shape<F>(select_shape, [&](auto s) { decltype(s)::launch(st, a, tau, n_sms); });
+        MergeShape<F, 256, 4>::launch(st, a, tau, n_sms);
     }
-    k_finish<F><<<(n * kGroup + kThreads - 1) / kThreads, kThreads, 0, st>>>(a);
+    launch_next(k_finish<F, false>, nb, kThreads, st, a);
+    if constexpr (sizeof(F) == 4) {
+        if (a.P.kappa_fp64 > 0.0f) launch_next(k_finish<F, true>, nb, kThreads, st, a);
+    }
     return cudaGetLastError();
+}
+
+// The resident grids of every shape, asked for outside any capture.
+template <class F, bool BWD> void prime_shapes_of(int n_sms) {
+    for (int q = 0; q < 6; ++q) with_move_shape<F, BWD>(q, [&](auto s) { decltype(s)::grid(n_sms); });
+    for (int q = 0; q < 3; ++q) with_find_shape<F>(q, [&](auto s) { decltype(s)::grid(n_sms); });
+    MergeShape<F, 256, 4>::grid(n_sms);
+}
+template <class F> void prime_shapes(int n_sms) {
+    prime_shapes_of<F, false>(n_sms);
+    if constexpr (sizeof(F) == 4) prime_shapes_of<F, true>(n_sms);
 }
 
 cudaError_t enqueue_rounds(cudaStream_t st, const BuildArgs& a, int n, int max_plan_len, int n_sms, int find_shape,
                            int select_shape, bool backward = false) {
-    // module hits loaded (their overlap trail exists): the module-aware kernels
-    const bool mod = a.w.otrail != nullptr;
-    if (backward)
-        return mod ? launch_rounds<float, true, true>(st, a, n, max_plan_len, n_sms, find_shape, select_shape)
-                   : launch_rounds<float, true>(st, a, n, max_plan_len, n_sms, find_shape, select_shape);
+    if (a.w.mod)   // module hits loaded
+        return launch_mod_rounds(st, a.geom, max_plan_len, a.P, a.H, a.S, a.out, a.w.mod, a.counters, n_sms, find_shape,
+                                 select_shape, backward);
+    if (backward) return launch_rounds<float, true>(st, a, n, max_plan_len, n_sms, find_shape, select_shape);
     // MKGB_FP64: the plain all-FP64 comparison path (same rounds, every Kalman step in FP64)
     if (a.P.precision == MKGB_FP64)
-        return mod ? launch_rounds<double, false, true>(st, a, n, max_plan_len, n_sms, find_shape, select_shape)
-                   : launch_rounds<double>(st, a, n, max_plan_len, n_sms, find_shape, select_shape);
-    return mod ? launch_rounds<float, false, true>(st, a, n, max_plan_len, n_sms, find_shape, select_shape)
-               : launch_rounds<float>(st, a, n, max_plan_len, n_sms, find_shape, select_shape);
+        return launch_rounds<double>(st, a, n, max_plan_len, n_sms, find_shape, select_shape);
+    return launch_rounds<float>(st, a, n, max_plan_len, n_sms, find_shape, select_shape);
 }
 
 bool capturable(cudaStream_t st) {
@@ -1487,19 +963,23 @@ bool capturable(cudaStream_t st) {
 
 }  // namespace
 
-size_t build_work_bytes(int n_seeds, int max_plan_len, int precision, bool with_ovl) {
-    return layout_build_work(nullptr, n_seeds, max_plan_len, precision == MKGB_FP64 ? 8 : 4, with_ovl, nullptr);
+size_t build_work_bytes(int n_seeds, int max_plan_len, int precision, bool modular) {
+    if (modular) return mod_work_bytes(n_seeds, max_plan_len, precision);
+    return layout_build_work(nullptr, n_seeds, max_plan_len, precision == MKGB_FP64 ? 8 : 4, nullptr);
 }
 
-BuildWork carve_build_work(void* base, int n_seeds, int max_plan_len, int precision, bool with_ovl) {
+BuildWork carve_build_work(void* base, int n_seeds, int max_plan_len, int precision, bool modular) {
     BuildWork w;
-    layout_build_work(static_cast<char*>(base), n_seeds, max_plan_len, precision == MKGB_FP64 ? 8 : 4, with_ovl,
-                      &w);
+    memset(&w, 0, sizeof(w));
+    if (modular)
+        w.mod = base;
+    else
+        layout_build_work(static_cast<char*>(base), n_seeds, max_plan_len, precision == MKGB_FP64 ? 8 : 4, &w);
     return w;
 }
 
-// The search of one call as a CUDA graph: the ~70 launches of the rounds (counters reset, k_start,
-// per plan step k_find, k_select and k_rescue, k_finish) are captured once and replayed while the
+// The search of one call as a CUDA graph: the ~90 launches of the rounds (counters reset, k_start,
+// per plan step k_move twice, k_find and k_merge, k_finish twice) are captured once and replayed while the
 // arguments, the launch shapes and the stream stay the same.
 struct BuildGraph {
     cudaGraphExec_t exec = nullptr;
@@ -1523,10 +1003,11 @@ cudaError_t launch_build(cudaStream_t st, const DevGeom* g, int max_plan_len, De
     if (S.n == 0) return cudaSuccess;
     BuildArgs a;
     memset(&a, 0, sizeof(a));   // padding included: the graph cache compares arguments bytewise
-    a.geom = g; a.P = P; a.H = H; a.S = S; a.out = out; a.w = w; a.counters = counters; a.max_steps = max_plan_len;
+    a.geom = g; a.P = P; a.H = H; a.S = S; a.out = out; a.w = w; a.counters = counters; a.slots = tile_slots(S.n);
     a.nfound0 = backward ? 0 : 3;
-    a.fused = find_shape >= 3 ? 1 : 0;
-    if (a.P.precision == MKGB_FP64)
+    if (w.mod)
+        prime_mod_shapes(a.P.precision, n_sms);
+    else if (a.P.precision == MKGB_FP64)
         prime_shapes<double>(n_sms);
     else
         prime_shapes<float>(n_sms);
