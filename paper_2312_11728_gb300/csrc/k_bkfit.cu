@@ -137,7 +137,9 @@ __global__ void __launch_bounds__(kThreads) k_bkfit(const DevGeom* __restrict__ 
     const int cnt = list ? *count : n;
     unsigned long long c_steps = 0, c_upd = 0;
     int c_newton = 0;
-    for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < cnt; r += gridDim.x * blockDim.x) {
+    // a list is dealt out to the SMs one by one, like every FP64 redo (k_fit.cu)
+    const int first = list ? blockIdx.x + gridDim.x * threadIdx.x : blockIdx.x * blockDim.x + threadIdx.x;
+    for (int r = first; r < cnt; r += gridDim.x * blockDim.x) {
         const int i = list ? list[r] : r;
         StateT<F> t;
         F sum;
@@ -187,7 +189,7 @@ cudaError_t launch_bkfit(cudaStream_t st, const DevGeom* g, DevParams P, const f
                                                 cov_scale, p_out, c_out, chi2_out, status_out, counters, rescue_list,
                                                 rescue_count, nullptr, nullptr);
     if (P.kappa_fp64 > 0.0f && rescue_list) {
-        const int rb = blocks < 2 * n_sms ? blocks : 2 * n_sms;
+        const int rb = n < 2 * n_sms ? n : 2 * n_sms;
         fit64<<<rb, kThreads, 0, st>>>(g, P, pay, n_hits, n, max_steps, layers, hits, p_start, c_start,
                                                  cov_scale, p_out, c_out, chi2_out, status_out, counters, nullptr,
                                                  nullptr, rescue_list, rescue_count);

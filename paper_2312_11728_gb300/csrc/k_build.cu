@@ -326,13 +326,16 @@ __global__ void __launch_bounds__(TH, MINB) k_move(BuildArgs a, int tau) {
     const int stride = gridDim.x * TH;
     // the descriptor of the next child is loaded one child ahead: it names the record to read
     const int4 none = make_int4(0, 0, 0, 0);
-    const int first = blockIdx.x * TH + threadIdx.x;
+    // the redo list is dealt out to the SMs one by one, like every FP64 redo (k_fit.cu)
+    const int lane0 = REDO ? blockIdx.x + gridDim.x * threadIdx.x : threadIdx.x;
+    const int base0 = REDO ? 0 : blockIdx.x * TH;
+    const int first = base0 + lane0;
     int sl_next = first < n ? list[first] : 0;
     int4 d_next = first < n ? a.w.child[slot_at(sl_next)] : none;
-    for (int base = blockIdx.x * TH; base < n; base += stride) {
+    for (int base = base0; base < n; base += stride) {
         // the warps of a block start a child together: they share the fetches of the loop's code
         __syncthreads();
-        const int idx = base + threadIdx.x;
+        const int idx = base + lane0;
         const int sl = sl_next;
         const int4 d = d_next;
         bool crossed = false;

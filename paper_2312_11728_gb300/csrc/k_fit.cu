@@ -126,6 +126,11 @@ __global__ void __launch_bounds__(kThreads) k_fit(const DevGeom* __restrict__ gp
 }
 
 // FP64 refit of the listed tracks (kappa rescue) or of all tracks (all-FP64 path, list == null).
+//
+// A list is dealt out to the blocks one by one, so that while it is short every item has a warp of its
+// own: the time is one track's chain of FP64 instructions (64 cycles each for a warp, whether one lane
+// is active or all), and lanes of other tracks only add their steps and branches to it.  1M tracks
+// with curling ones: 1.68 -> 1.62 ms.
 template <bool MOD>
 __global__ void __launch_bounds__(kThreads) k_fit64(const DevGeom* __restrict__ gp, DevParams P,
                                                     const float4* __restrict__ pay, int64_t n_hits, int n,
@@ -140,7 +145,8 @@ __global__ void __launch_bounds__(kThreads) k_fit64(const DevGeom* __restrict__ 
     const int cnt = list ? *count : n;
     unsigned long long c_steps = 0, c_upd = 0;
     int c_newton = 0;
-    for (int r = blockIdx.x * blockDim.x + threadIdx.x; r < cnt; r += gridDim.x * blockDim.x) {
+    const int first = list ? blockIdx.x + gridDim.x * threadIdx.x : blockIdx.x * blockDim.x + threadIdx.x;
+    for (int r = first; r < cnt; r += gridDim.x * blockDim.x) {
         const int i = list ? list[r] : r;
         StateT<double> t;
         double sum;
@@ -241,7 +247,7 @@ cudaError_t launch_fit(cudaStream_t st, const DevGeom* g, DevParams P, const flo
     fit<<<blocks, kThreads, 0, st>>>(g, P, pay, n_hits, n, max_steps, layers, hits, p0, c0, p_out, c_out, chi2_out,
                                     status_out, counters, rescue_list, rescue_count);
     if (P.kappa_fp64 > 0.0f && rescue_list) {
-        const int rb = blocks < 2 * n_sms ? blocks : 2 * n_sms;
+        const int rb = n < 2 * n_sms ? n : 2 * n_sms;
         fit64<<<rb, kThreads, 0, st>>>(g, P, pay, n_hits, n, max_steps, layers, hits, p0, c0, p_out, c_out,
                                       chi2_out, status_out, counters, rescue_list, rescue_count);
     }
