@@ -80,7 +80,7 @@ struct mkgb_ctx {
     int n_events = 0, n_layers = 0;
     int64_t n_hits = 0;
     std::vector<int64_t> seg_off_h;
-    DevBuf seg_off, in_xyz, in_cov, pay, ep_tmp, bin_of_hit, hit_seg, bins, hb_ep, hb_pay, cursor, scan_tmp;
+    DevBuf seg_off, in_xyz, in_cov, pay, place, hit_seg, bins, hb_ep, hb_pay, scan_tmp;
     int n_seeds = 0;
     DevBuf seed_hits, seed_state, seed_state64, seed_info, seed_key, key_counts, key_cursor, seed_order, seed_scan_tmp;
     DevBuf seed_redo;   // the seeds whose mixed-precision fit is redone in FP64: count, then indices
@@ -125,6 +125,7 @@ HitStore hit_store(const mkgb_ctx* c) {
     H.n_layers = c->n_layers;
     H.n_hits = c->n_hits;
     H.pay = (const float4*)c->pay.p;
+    H.hb = (const float4*)c->hb_pay.p;
     H.hb_ep = (const float2*)c->hb_ep.p;
     H.hb_pay = (const float4*)c->hb_pay.p;
     H.bin_start = (const int*)c->bins.p;
@@ -306,8 +307,8 @@ void mkgb_destroy(mkgb_ctx* ctx) {
         if (ctx->ev_seedin) cudaEventDestroy(ctx->ev_seedin);
         if (ctx->ev_fitin) cudaEventDestroy(ctx->ev_fitin);
         if (ctx->ev_start) cudaEventDestroy(ctx->ev_start);
-        DevBuf* all[] = {&ctx->host_run, &ctx->geom_d, &ctx->seg_off, &ctx->in_xyz, &ctx->in_cov, &ctx->pay, &ctx->ep_tmp,
-                         &ctx->bin_of_hit, &ctx->hit_seg, &ctx->bins, &ctx->hb_ep, &ctx->hb_pay, &ctx->cursor,
+        DevBuf* all[] = {&ctx->host_run, &ctx->geom_d, &ctx->seg_off, &ctx->in_xyz, &ctx->in_cov, &ctx->pay, &ctx->place,
+                         &ctx->hit_seg, &ctx->bins, &ctx->hb_ep, &ctx->hb_pay,
                          &ctx->scan_tmp, &ctx->seed_hits, &ctx->seed_state, &ctx->seed_state64, &ctx->seed_info, &ctx->seed_key,
                          &ctx->key_counts, &ctx->key_cursor, &ctx->seed_order, &ctx->seed_scan_tmp, &ctx->seed_redo,
                          &ctx->counters_build, &ctx->counters_fit, &ctx->queue, &ctx->rescue_list,
@@ -522,13 +523,12 @@ int load_hits_impl(mkgb_ctx* ctx, int n_events, const int64_t* seg_off, const fl
         dc = (const float*)ctx->in_cov.p;
     }
     CK(ensure(ctx->pay, 48 * n));
-    CK(ensure(ctx->ep_tmp, 8 * n));
-    CK(ensure(ctx->bin_of_hit, 4 * n));
+    CK(ensure(ctx->place, 16 * n));
     CK(ensure(ctx->hit_seg, 4 * n));
-    CK(ensure(ctx->hb_ep, 8 * n));
-    CK(ensure(ctx->hb_pay, 48 * n));
+    const bool modular = hit_module != nullptr && n > 0;
+    if (modular) CK(ensure(ctx->hb_ep, 8 * n));
+    CK(ensure(ctx->hb_pay, (modular ? 48 : 16) * n));   // the payload, or (eta, phi, id) without module hits
     CK(ensure(ctx->bins, 4 * (nbins + 1)));
-    CK(ensure(ctx->cursor, 4 * (nbins + 1)));
     CK(ensure(ctx->scan_tmp, 4 * scan_tmp_ints(nbins + 1)));
     const int* dm = hit_module;
     if (hit_module && !on_device && n > 0) {
@@ -542,8 +542,8 @@ int load_hits_impl(mkgb_ctx* ctx, int n_events, const int64_t* seg_off, const fl
             CK(cudaStreamWaitEvent(st, chunks->ready[k], 0));
             CK(launch_hit_prep(st, (const DevGeom*)ctx->geom_d.p, L, (const int64_t*)ctx->seg_off.p, (int)nseg, n, dx,
                                dc, n > 0 ? dm : nullptr, ctx->geom_h.bins_per_event, (float4*)ctx->pay.p,
-                               (float2*)ctx->ep_tmp.p, (int*)ctx->bin_of_hit.p, (int*)ctx->hit_seg.p,
-                               (int*)ctx->bins.p, chunks->hit_off[k], chunks->hit_off[k + 1]));
+                               (int4*)ctx->place.p, (int*)ctx->hit_seg.p, (int*)ctx->bins.p, chunks->hit_off[k],
+                               chunks->hit_off[k + 1]));
             if (chunks->after) {
                 const int rc = chunks->after(k);
                 if (rc != MKGB_OK) return rc;
@@ -552,7 +552,7 @@ int load_hits_impl(mkgb_ctx* ctx, int n_events, const int64_t* seg_off, const fl
     } else {
         CK(launch_hit_prep(st, (const DevGeom*)ctx->geom_d.p, L, (const int64_t*)ctx->seg_off.p, (int)nseg, n, dx, dc,
                            n > 0 ? dm : nullptr, ctx->geom_h.bins_per_event, (float4*)ctx->pay.p,
-                           (float2*)ctx->ep_tmp.p, (int*)ctx->bin_of_hit.p, (int*)ctx->hit_seg.p, (int*)ctx->bins.p));
+                           (int4*)ctx->place.p, (int*)ctx->hit_seg.p, (int*)ctx->bins.p));
     }
     ctx->has_hits = false;
     if (hit_module && n > 0) {   // every module id must fit its hit's layer (synchronises)
@@ -570,10 +570,8 @@ int load_hits_impl(mkgb_ctx* ctx, int n_events, const int64_t* seg_off, const fl
     CK(cudaEventRecord(ctx->ev_prep, st));
     CK(cudaStreamWaitEvent(ctx->aux, ctx->ev_prep, 0));
     CK(exclusive_scan(ctx->aux, (const int*)ctx->bins.p, (int*)ctx->bins.p, nbins, (int*)ctx->scan_tmp.p));
-    CK(cudaMemcpyAsync(ctx->cursor.p, ctx->bins.p, 4 * nbins, cudaMemcpyDeviceToDevice, ctx->aux));
-    CK(launch_hit_scatter(ctx->aux, n, (const float4*)ctx->pay.p, (const float2*)ctx->ep_tmp.p,
-                          (const int*)ctx->bin_of_hit.p, (int*)ctx->cursor.p, (float2*)ctx->hb_ep.p,
-                          (float4*)ctx->hb_pay.p));
+    CK(launch_hit_scatter(ctx->aux, n, (const int4*)ctx->place.p, (const int*)ctx->bins.p, (const float4*)ctx->pay.p,
+                          modular, (float4*)ctx->hb_pay.p, (float2*)ctx->hb_ep.p, (float4*)ctx->hb_pay.p));
     CK(cudaEventRecord(ctx->ev_bins, ctx->aux));
     ctx->bins_pending = true;
     if (!on_device) CK(cudaStreamSynchronize(st));
@@ -581,7 +579,7 @@ int load_hits_impl(mkgb_ctx* ctx, int n_events, const int64_t* seg_off, const fl
     ctx->n_hits = n;
     ctx->has_hits = true;
     ctx->has_seeds = false;
-    ctx->mod_hits = hit_module != nullptr && n > 0;
+    ctx->mod_hits = modular;
     return MKGB_OK;
 }
 

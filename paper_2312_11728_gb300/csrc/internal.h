@@ -21,8 +21,9 @@ struct HitStore {
     int n_events, n_layers;
     int64_t n_hits;
     const float4* pay;         // 3 float4 per hit, original order: (x,y,z,id) (v0..v3) (v4,v5,-,-)
-    const float2* hb_ep;       // binned order: (eta, phi)
-    const float4* hb_pay;      // binned order payload
+    const float4* hb;          // binned order: (eta, phi, id, -); without module hits
+    const float2* hb_ep;       // binned order: (eta, phi), with module hits
+    const float4* hb_pay;      // binned order payload, with module hits
     const int* bin_start;      // E*bins_per_event + 1 offsets into the binned arrays
     const int* hit_seg;        // per hit: segment e*L + l
 };
@@ -65,7 +66,7 @@ struct BuildWork {
     int* seeds[2];    // work list of seeds with a live candidate per round
     int4* sinfo;      // per ordered seed: (plan position of its first step, first step, steps, event)
     int* fin;         // per ordered seed: rounds searched, -1 none
-    int* trail;       // per round and slot ((code + 4) << 3 | parent slot); a hit's code is its binned index
+    int* trail;       // per round and slot ((code + 4) << 3 | parent slot); code: the hit's id or MKGB_HIT_*
     int* redo;        // children of the round whose update is redone in FP64
     int* found;       // candidates of the round that crossed their layer
     int* counts;      // [live0, live1, seeds0, seeds1, redo, found]
@@ -80,14 +81,15 @@ constexpr int kNumCounters = 5;
 // hits [h0, h1) (h1 < 0: up to n_hits), so that a batch arriving in chunks is prepared per chunk.
 cudaError_t launch_hit_prep(cudaStream_t st, const DevGeom* g, int n_layers, const int64_t* seg_off, int n_seg,
                             int64_t n_hits, const float* xyz, const float* cov, const int* hit_mod,
-                            int bins_per_event, float4* pay, float2* ep_tmp, int* bin_of_hit, int* hit_seg,
-                            int* counts, int64_t h0 = 0, int64_t h1 = -1);
+                            int bins_per_event, float4* pay, int4* place, int* hit_seg, int* counts, int64_t h0 = 0,
+                            int64_t h1 = -1);
 // Counts into *bad the hits whose module does not fit their layer (a module hit on a layer without
 // modules or on another layer's module, a hit without module on a modular layer, an index out of range).
 cudaError_t launch_check_modules(cudaStream_t st, const DevGeom* g, int n_layers, int64_t n_hits,
                                  const int* hit_seg, const int* hit_mod, int* bad);
-cudaError_t launch_hit_scatter(cudaStream_t st, int64_t n_hits, const float4* pay, const float2* ep_tmp,
-                               const int* bin_of_hit, int* cursor, float2* hb_ep, float4* hb_pay);
+// The binned hits: hb, or with module hits hb_ep and hb_pay (HitStore).
+cudaError_t launch_hit_scatter(cudaStream_t st, int64_t n_hits, const int4* place, const int* bin_start,
+                               const float4* pay, bool modular, float4* hb, float2* hb_ep, float4* hb_pay);
 // Exclusive scan of n ints (out[n] gets the total); tmp must hold scan_tmp_ints(n) ints.
 size_t scan_tmp_ints(int64_t n);
 cudaError_t exclusive_scan(cudaStream_t st, const int* in, int* out, int64_t n, int* tmp);

@@ -204,8 +204,8 @@ struct BuildArgs {
     int nfound0;     // hits a track has when its search starts (3 seed hits forwards, 0 backwards)
 };
 
-// Child descriptor (one int4 per slot): parent slot | kind << 4 | disk << 8, the binned index of its
-// hit (K_HIT) or the seed (K_SEED), its score, its missed layers.  disk: the parent's prediction lies
+// Child descriptor (one int4 per slot): parent slot | kind << 4 | disk << 8, its hit (K_HIT) or the
+// seed (K_SEED), its score, its missed layers.  disk: the parent's prediction lies
 // on a disk.
 __device__ __forceinline__ int4 pack_child(int parent, int kind, bool disk, int q, float score, int nholes) {
     return make_int4(parent | (kind << 4) | ((int)disk << 8), q, __float_as_int(score), nholes);
@@ -255,7 +255,7 @@ __global__ void __launch_bounds__(kThreads) k_start(BuildArgs a) {
 
 // The update of a child redone in FP64 from its parent's FP32 prediction, narrowed (mixed
 // precision, growth G3).  False: the update failed.
-__device__ __noinline__ bool update_fp64(int surface, const Pred& pq, const float4* __restrict__ hb_pay, int hq,
+__device__ __noinline__ bool update_fp64(int surface, const Pred& pq, const float4* __restrict__ pay, int id,
                                          State& t) {
     PredT<double> qd;
     qd.xh = pq.xh; qd.yh = pq.yh; qd.zh = pq.zh; qd.xl = pq.xl; qd.yl = pq.yl; qd.zl = pq.zl;
@@ -263,7 +263,7 @@ __device__ __noinline__ bool update_fp64(int surface, const Pred& pq, const floa
 #pragma unroll
     for (int q = 0; q < 15; ++q) qd.c[q] = pq.c[q];
     double m[3], v[6];
-    load_hit(hb_pay, hq, m, v, nullptr);
+    load_hit(pay, id, m, v, nullptr);
     StateT<double> td;
     const bool ok = kalman_update(surface, qd, m[0], m[1], m[2], v, td);
     if (ok) narrow_state(td, t);
@@ -350,7 +350,7 @@ __global__ void __launch_bounds__(TH, MINB) k_move(BuildArgs a, int tau) {
                 load_seed_rec(seed_states<F>(a.S) + (int64_t)d.y * kSeedStateStride, f);
             else
                 load_rec<F, kStateWords>(prev, (sl & ~(kGroup - 1)) | child_parent(d), f);
-            if (child_kind(d) == K_HIT) load_hit(a.H.hb_pay, d.y, m, v, nullptr);
+            if (child_kind(d) == K_HIT) load_hit(a.H.pay, d.y, m, v, nullptr);
             if (idx + (int64_t)stride < n) {
                 sl_next = list[idx + stride];
                 d_next = a.w.child[slot_at(sl_next)];
@@ -358,7 +358,7 @@ __global__ void __launch_bounds__(TH, MINB) k_move(BuildArgs a, int tau) {
             if constexpr (REDO) {
                 Pred pq;
                 unpack_pred(f, pq);
-                fail = update_fp64(child_surface(d), pq, a.H.hb_pay, d.y, t) ? 0 : 3;
+                fail = update_fp64(child_surface(d), pq, a.H.pay, d.y, t) ? 0 : 3;
             } else {
                 fail = child_state(a, d, f, m, v, t);
             }
@@ -406,8 +406,7 @@ __global__ void __launch_bounds__(TH, MINB) k_find(BuildArgs a, int tau) {
     // per-thread sorted list of hit children (chi2 asc, id asc), one column per thread
     __shared__ float s_x2[kGroup][TH];
     __shared__ int s_id[kGroup][TH];
-    __shared__ int s_hq[kGroup][TH];
-    __shared__ int s_q[kQueue][TH];   // hits inside the window, waiting for their chi2
+    __shared__ int s_q[kQueue][TH];   // ids of the hits inside the window, waiting for their chi2
     next_kernel_may_start();
     load_geom_smem(a.geom, g);
     wait_for_last_kernel();
@@ -458,7 +457,7 @@ __global__ void __launch_bounds__(TH, MINB) k_find(BuildArgs a, int tau) {
             q0 = __ldg(a.H.bin_start + at);
             q1 = __ldg(a.H.bin_start + at + ((rg & (nr - 1)) ? run2 : run1));
         };
-        auto inside = [&](const float2& ep) {
+        auto inside = [&](const float4& ep) {
             return fabs(F(ep.x) - w.eta) <= w.deta && fabs(wrap_pi(F(ep.y) - w.phi)) <= w.dphi;
         };
         int rg = 0, hq = 0, q1 = 0, hq_next = 0, q1_next = 0;
@@ -477,19 +476,18 @@ __global__ void __launch_bounds__(TH, MINB) k_find(BuildArgs a, int tau) {
                     continue;
                 }
                 const bool two = hq + 1 < q1 && nq + 1 < kQueue;
-                const float2 ep0 = __ldg(a.H.hb_ep + hq), ep1 = __ldg(a.H.hb_ep + hq + (int)two);
+                const float4 ep0 = __ldg(a.H.hb + hq), ep1 = __ldg(a.H.hb + hq + (int)two);
                 c_tested += 1 + two;
-                if (inside(ep0)) s_q[nq++][tx] = hq;
-                if (two && inside(ep1)) s_q[nq++][tx] = hq + 1;
+                if (inside(ep0)) s_q[nq++][tx] = __float_as_int(ep0.z);
+                if (two && inside(ep1)) s_q[nq++][tx] = __float_as_int(ep1.z);
                 hq += 1 + two;
             }
             c_chi2 += nq;
             for (int jq = 0; jq < nq; ++jq) {
-                const int h = s_q[jq][tx];
+                const int id = s_q[jq][tx];
                 F mh[3], vh[6];
-                int id;
                 F x2f;
-                load_hit(a.H.hb_pay, h, mh, vh, &id);
+                load_hit(a.H.pay, id, mh, vh, nullptr);
                 const bool okx = chi2_hit(fr, q, mh[0], mh[1], mh[2], vh, x2f);
                 if (!okx || !(x2f < F(P.chi2_cut))) continue;
                 const float x2 = float(x2f);   // scores and child order in FP32
@@ -499,12 +497,10 @@ __global__ void __launch_bounds__(TH, MINB) k_find(BuildArgs a, int tau) {
                 while (j > 0 && (x2 < s_x2[j - 1][tx] || (x2 == s_x2[j - 1][tx] && id < s_id[j - 1][tx]))) {
                     s_x2[j][tx] = s_x2[j - 1][tx];
                     s_id[j][tx] = s_id[j - 1][tx];
-                    s_hq[j][tx] = s_hq[j - 1][tx];
                     --j;
                 }
                 s_x2[j][tx] = x2;
                 s_id[j][tx] = id;
-                s_hq[j][tx] = h;
                 if (n_h < kGroup) ++n_h;
             }
         }
@@ -512,9 +508,9 @@ __global__ void __launch_bounds__(TH, MINB) k_find(BuildArgs a, int tau) {
         int4* lrec = a.w.ls + word_at<2>(sl, 0);
         lrec[0] = make_int4(n_h | (L.kind == MKGB_DISK ? kDiskBit : 0), nh_kind, __float_as_int(nh_score), 0);
         for (int j = 0; j < n_h; j += 2) {
-            const int4 e = make_int4(__float_as_int(s_x2[j][tx]), s_hq[j][tx],
+            const int4 e = make_int4(__float_as_int(s_x2[j][tx]), s_id[j][tx],
                                      __float_as_int(j + 1 < n_h ? s_x2[j + 1][tx] : kBig),
-                                     j + 1 < n_h ? s_hq[j + 1][tx] : 0);
+                                     j + 1 < n_h ? s_id[j + 1][tx] : 0);
             if (j == 0)
                 lrec[kTile * kGroup] = e;
             else
@@ -576,7 +572,7 @@ __global__ void __launch_bounds__(TH, MINB) k_merge(BuildArgs a, int tau) {
         const float nh_score = stopped ? score : __int_as_float(e0.z);
         const bool disk = (e0.x & kDiskBit) != 0;
         const bool has_nh = nh_kind != K_NONE;
-        auto hit_entry = [&](int j) {   // (chi2, binned index) of the parent's j-th hit
+        auto hit_entry = [&](int j) {   // (chi2, id) of the parent's j-th hit
             if (j == 0) return make_int2(e1.x, e1.y);
             if (j == 1) return make_int2(e1.z, e1.w);
             return reinterpret_cast<const int2*>(a.w.ls_more + word_at<3>(sl, j / 2 - 1))[j & 1];
@@ -715,14 +711,14 @@ __global__ void __launch_bounds__(kThreads) k_finish(BuildArgs a) {
         } else {
             d = a.w.child[slot_at(cs)];
             load_rec<F, kStateWords>(a.w.rec[(rounds & 1) ^ 1], i * kGroup + child_parent(d), f);
-            if (child_kind(d) == K_HIT) load_hit(a.H.hb_pay, d.y, m, v, nullptr);
+            if (child_kind(d) == K_HIT) load_hit(a.H.pay, d.y, m, v, nullptr);
         }
         int fail = child_state(a, d, f, m, v, t);
         if (fail == 2) {
             if constexpr (REDO) {
                 Pred q;
                 unpack_pred(f, q);
-                fail = update_fp64(child_surface(d), q, a.H.hb_pay, d.y, t) ? 0 : 1;
+                fail = update_fp64(child_surface(d), q, a.H.pay, d.y, t) ? 0 : 1;
             } else {
                 a.w.redo[atomicAdd(a.w.counts + 4, 1)] = i;
                 return;
@@ -748,8 +744,8 @@ __global__ void __launch_bounds__(kThreads) k_finish(BuildArgs a) {
         for (int tau = min(rounds, si.z) - 1; tau >= 0; --tau) {
             const int64_t at = (int64_t)tau * a.slots + slot_at(i * kGroup + s_);
             const int v = a.w.trail[at];
-            const int code = (v >> 3) - 4;   // a hit: its binned index
-            hrow[si.y + tau] = code >= 0 ? __float_as_int(__ldg(a.H.hb_pay + 3 * (int64_t)code).w) : code;
+            const int code = (v >> 3) - 4;
+            hrow[si.y + tau] = code;
             s_ = v & 7;
         }
     } else {
