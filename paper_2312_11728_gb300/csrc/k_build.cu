@@ -21,8 +21,8 @@
 // merge and update by eight lanes per seed, 18.5 of 32 lanes active, states and predictions both
 // written, records one after another) took 21.6 ms for 64 Phase-2-like events (1.28M seeds, 58M
 // crossed steps) and 0.90 ms for one; one kernel for update, propagation and window 17.2 ms (its 128
-// registers also held the window's chains of loads to 16 warps); these three 15.9 and 0.66 ms:
-// k_move 7.4 ms, k_find 2.9, k_merge 4.8 of the 64 events.  k_move is bound by issue and latency
+// registers also held the window's chains of loads to 16 warps); these three 15.8 and 0.65 ms:
+// k_move 7.5 ms, k_find 3.1, k_merge 4.3 of the 64 events.  k_move is bound by issue and latency
 // together (47% issue active, 28% of DRAM), k_find and k_merge by their dependent loads.
 //
 // No kernel waits on another block; every loop is bounded by a list length, a window's bin range or
@@ -526,7 +526,7 @@ __global__ void __launch_bounds__(TH, MINB) k_find(BuildArgs a, int tau) {
 // slot, then place in the parent's list) into shared memory and counts the keys above its own: that
 // count is its slot among the N best, so a parent's lane writes its kept children straight from its
 // registers, with no exchange of their contents and no round per rank. 
-// 64 events: 4.8 ms; eight lanes exchanging keys and contents by shuffles, a round per rank: 7.4 ms;
+// 64 events: 4.3 ms (4.8 with a walk over the keys per child); eight lanes exchanging keys and contents by shuffles, a round per rank: 7.4 ms;
 // one thread per seed with its eight best in registers: 3.8 ms, but 1.3 times the whole search of one
 // event (0.86 against 0.66 ms), where the latency of a thread's serial lists counts.
 constexpr int kNoHit = 15;   // place of the child without a hit
@@ -563,7 +563,11 @@ __global__ void __launch_bounds__(TH, MINB) k_merge(BuildArgs a, int tau) {
         const int sl = i * kGroup + slot;
         // all of the slot's words at once (those of an empty slot are not used)
         const int4 mt = a.w.meta[cur][slot_at(sl)];
-        const int4 e0 = a.w.ls[word_at<2>(sl, 0)], e1 = a.w.ls[word_at<2>(sl, 1)];
+        int4 e0 = make_int4(0, K_NONE, 0, 0), e1 = e0;
+        if (mt.w != 0) {
+            e0 = a.w.ls[word_at<2>(sl, 0)];
+            e1 = a.w.ls[word_at<2>(sl, 1)];
+        }
         const float score = __int_as_float(mt.x);
         const bool alive = gact && mt.w != 0, stopped = ((mt.z >> 16) & 1) != 0;
         const bool searched = alive && !stopped;
@@ -591,22 +595,29 @@ __global__ void __launch_bounds__(TH, MINB) k_merge(BuildArgs a, int tau) {
         for (int j = 0; j < n_h; ++j) keys[end - cnt + j] = child_key(hit_score(j), slot, j);
         if (has_nh) keys[end - 1] = child_key(nh_score, slot, kNoHit);
         __syncwarp();
-        auto rank_of = [&](unsigned long long k) {
-            int r = 0;
-            for (int q = 0; q < total; ++q) r += keys[q] > k;
-            return r;
-        };
+        // most parents have one hit child and one without: both are ranked in one walk over the keys
+        const unsigned long long k_first = n_h > 0 ? keys[end - cnt] : ~0ull, k_nh = has_nh ? keys[end - 1] : ~0ull;
+        int r_first = 0, nh_slot = 0;
+        for (int q = 0; q < total; ++q) {
+            const unsigned long long k = keys[q];
+            r_first += k > k_first;
+            nh_slot += k > k_nh;
+        }
         int kept_hits = 0;         // the first of the parent's hits are kept, at these slots (4 bits each)
         unsigned hit_slots = 0, kept = 0, live = 0;
         for (int j = 0; j < n_h; ++j) {
-            const int r = rank_of(keys[end - cnt + j]);
+            int r = r_first;
+            if (j > 0) {
+                const unsigned long long kj = keys[end - cnt + j];
+                r = 0;
+                for (int q = 0; q < total; ++q) r += keys[q] > kj;
+            }
             if (r >= P.max_cands) break;   // the others come after it
             hit_slots |= (unsigned)r << (4 * j);
             live |= 1u << r;
             ++kept_hits;
         }
         c_upd += kept_hits;
-        const int nh_slot = has_nh ? rank_of(keys[end - 1]) : kGroup;
         const bool nh_kept = nh_slot < P.max_cands && has_nh;
         const bool nh_stop = nh_kept && nh_kind == K_STOP;
         kept = live | (nh_kept ? 1u << nh_slot : 0u);

@@ -18,7 +18,7 @@
 // k_start fills round 0 from the seed states; k_finish picks each seed's best candidate and walks
 // the trail back for its hit list (a13).
 //
-// Batches without module hits go through the rounds of k_build.cu, which are faster there (15.9
+// Batches without module hits go through the rounds of k_build.cu, which are faster there (15.8
 // against 21.6 ms for 64 events).  With module hits those rounds were 5% faster than these (0.92
 // against 0.97 ms, 12,000 seeds of two events): the step to a module's plane takes most of the time,
 // a call with its own stack either way.  But their compiled Newton loop rounds some crossings of the
