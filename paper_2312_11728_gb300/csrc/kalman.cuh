@@ -467,7 +467,9 @@ __device__ __forceinline__ void material_cov(G qc[15], F th02, F kc, F st, F a) 
 // path length solved in a lower precision (the FP64 steps then need one or two iterations);
 // s_out returns the path length; mat_fp32 computes the material terms (Highland angle, energy-
 // loss factor: small corrections, ~1e-7 relative in FP32) in FP32 for an FP64 step.
-template <class F, class G, bool BACKWARD = false>
+// SPARSE: cin couples positions with positions only and k, phi and theta with nothing (the state after
+// a seed's first update): the products with its zeros are left out, which changes no result.
+template <class F, class G, bool BACKWARD = false, bool SPARSE = false>
 __device__ __forceinline__ int propagate_core(const DevLayer& L, float cBf, int material, const StateT<F>& t,
                                               const G cin[21], PredT<F>& q, G qc[15], int& newton_it,
                                               F* dir = nullptr, const F* xscale = nullptr,
@@ -689,7 +691,8 @@ __device__ __forceinline__ int propagate_core(const DevLayer& L, float cBf, int 
         for (int j = 0; j < 6; ++j) {
             G acc = G(0);
 #pragma unroll
-            for (int l = 0; l < 6; ++l) acc = fma(G(J[r][l]), cin[ix(l, j)], acc);
+            for (int l = 0; l < 6; ++l)
+                if (!SPARSE || (j < 3 ? l < 3 : l == j)) acc = fma(G(J[r][l]), cin[ix(l, j)], acc);
             T[r][j] = acc;
         }
 #pragma unroll

@@ -104,7 +104,11 @@ __device__ __forceinline__ bool seed_fit(const DevGeom& g, const DevParams& P, c
             narrow_to_fp32(t, t32);
             Pred q32;
             float d32[4];
-            ok = ok && propagate_core<float, F>(L, g.cB, P.material, t32, t.c, q32, q.c, newton, d32) == 1;
+            // (144 of the ~1,870 FP64 operations of a seed are the first step's products with zeros)
+            if (j == 1)
+                ok = ok && propagate_core<float, F, false, true>(L, g.cB, P.material, t32, t.c, q32, q.c, newton, d32) == 1;
+            else
+                ok = ok && propagate_core<float, F>(L, g.cB, P.material, t32, t.c, q32, q.c, newton, d32) == 1;
             q.xh = F(q32.xh); q.yh = F(q32.yh); q.zh = F(q32.zh);
             q.xl = F(q32.xl); q.yl = F(q32.yl); q.zl = F(q32.zl);
             q.k = F(q32.k); q.phi = F(q32.phi); q.pl = F(q32.pl); q.th = F(q32.th); q.tl = F(q32.tl);
