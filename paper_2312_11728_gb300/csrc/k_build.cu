@@ -54,6 +54,8 @@ template <class F> struct Vec16;
 template <> struct Vec16<float> { using T = float4; };
 template <> struct Vec16<double> { using T = double2; };
 
+__device__ __forceinline__ void prefetch_l2(const void* p) { asm volatile("prefetch.global.L2 [%0];" ::"l"(p)); }
+
 // Slots are laid out in tiles of 32 seeds: the 16-byte words of an array run over the seeds of a tile,
 // then over the eight slots, then over the words of a record.  A warp of k_move or k_merge, whose slots
 // come from a few neighbouring seeds, then touches about eight 128-byte lines per 16-byte load; with
@@ -366,6 +368,14 @@ __global__ void __launch_bounds__(TH, MINB) k_move(BuildArgs a, int tau) {
         // children with and without a hit go on together (without this the compiler makes a copy of
         // the rest for each kind: 17.7 of 32 lanes active instead of 28)
         __syncwarp();
+        // the next child's record and hit on their way to the L2 (64-event search 15.8 -> 15.45 ms)
+        if (!REDO && idx + (int64_t)stride < n && child_kind(d_next) != K_SEED) {
+            const char* r = reinterpret_cast<const char*>(prev) +
+                            16 * word_at<rec_vecs<F>()>((sl_next & ~(kGroup - 1)) | child_parent(d_next), 0);
+#pragma unroll
+            for (int j = 0; j < rec_vecs<F>(); ++j) prefetch_l2(r + 16 * j * (kTile * kGroup));
+            if (child_kind(d_next) == K_HIT) prefetch_l2(a.H.pay + 3 * (int64_t)d_next.y);
+        }
         int nh_kind = K_NONE;
         if (fail == 0) {
             const DevLayer& L = g.layers[g.plan[si.x + tau]];
