@@ -84,7 +84,7 @@ struct mkgb_ctx {
     int n_seeds = 0;
     DevBuf seed_hits, seed_state, seed_state64, seed_info, seed_key, key_counts, key_cursor, seed_order, seed_scan_tmp;
     DevBuf seed_redo;   // the seeds whose mixed-precision fit is redone in FP64: count, then indices
-    DevBuf counters_build, counters_fit, queue, rescue_list, rescue_count, build_work, probe_sink, grad_ck;
+    DevBuf counters_build, counters_fit, queue, rescue_list, rescue_count, build_work, probe_sink, grad_ck, fit_order;
     // backward search: the geometry with reversed plans and the tracks' start records
     DevBuf geom_bwd_d, bw_state, bw_info, bw_order;
     DevBuf clean_scratch;   // seed cleaning / duplicate removal index
@@ -312,7 +312,7 @@ void mkgb_destroy(mkgb_ctx* ctx) {
                          &ctx->scan_tmp, &ctx->seed_hits, &ctx->seed_state, &ctx->seed_state64, &ctx->seed_info, &ctx->seed_key,
                          &ctx->key_counts, &ctx->key_cursor, &ctx->seed_order, &ctx->seed_scan_tmp, &ctx->seed_redo,
                          &ctx->counters_build, &ctx->counters_fit, &ctx->queue, &ctx->rescue_list,
-                         &ctx->rescue_count, &ctx->build_work, &ctx->probe_sink, &ctx->grad_ck,
+                         &ctx->rescue_count, &ctx->build_work, &ctx->probe_sink, &ctx->grad_ck, &ctx->fit_order,
                          &ctx->geom_bwd_d, &ctx->bw_state, &ctx->bw_info, &ctx->bw_order,
                          &ctx->clean_scratch, &ctx->mods_d, &ctx->in_mod, &ctx->mod_bad};
         for (DevBuf* b : all) release(*b);
@@ -820,11 +820,17 @@ int mkgb_fit(mkgb_ctx* ctx, int n, int max_steps, const int32_t* layers, const i
     CK(ensure(ctx->rescue_list, 4 * (N > 0 ? N : 1)));
     CK(ensure(ctx->rescue_count, 16));
     CK(cudaMemsetAsync(ctx->rescue_count.p, 0, 16, st));
+    const int* order = nullptr;
+    const size_t ob = ctx->params.precision == MKGB_FP64 ? 0 : fit_order_bytes(n, max_steps);
+    if (ob > 0) {
+        CK(ensure(ctx->fit_order, ob));
+        CK(launch_fit_order(st, (const DevGeom*)ctx->geom_d.p, n, max_steps, (const int*)dl, ctx->fit_order.p, &order));
+    }
     CK(launch_fit(st, (const DevGeom*)ctx->geom_d.p, ctx->params, (const float4*)ctx->pay.p,
                   ctx->has_hits ? ctx->n_hits : 0, n, max_steps, (const int*)dl, (const int*)dh, (const float*)dp0,
                   (const float*)dc0, (float*)po, (float*)co, (float*)xo, (int*)so,
                   (unsigned long long*)ctx->counters_fit.p, (int*)ctx->rescue_list.p, (int*)ctx->rescue_count.p,
-                  ctx->n_sms, ctx->mod_hits));
+                  ctx->n_sms, ctx->mod_hits, order));
     CK(copy_back(ctx, p_out, po, 24 * N, on_device));
     CK(copy_back(ctx, c_out, co, 84 * N, on_device));
     CK(copy_back(ctx, chi2_out, xo, 4 * N, on_device));
@@ -866,11 +872,17 @@ int mkgb_fit_backward(mkgb_ctx* ctx, int n, int max_steps, const int32_t* layers
     CK(ensure(ctx->rescue_list, 4 * (N > 0 ? N : 1)));
     CK(ensure(ctx->rescue_count, 16));
     CK(cudaMemsetAsync(ctx->rescue_count.p, 0, 16, st));
+    const int* order = nullptr;
+    const size_t ob = ctx->params.precision == MKGB_FP64 ? 0 : fit_order_bytes(n, max_steps);
+    if (ob > 0) {
+        CK(ensure(ctx->fit_order, ob));
+        CK(launch_fit_order(st, (const DevGeom*)ctx->geom_d.p, n, max_steps, (const int*)dl, ctx->fit_order.p, &order));
+    }
     CK(launch_bkfit(st, (const DevGeom*)ctx->geom_d.p, ctx->params, (const float4*)ctx->pay.p,
                     ctx->has_hits ? ctx->n_hits : 0, n, max_steps, (const int*)dl, (const int*)dh, (const float*)dp0,
                     (const float*)dc0, cov_scale, (float*)po, (float*)co, (float*)xo, (int*)so,
                     (unsigned long long*)ctx->counters_fit.p, (int*)ctx->rescue_list.p, (int*)ctx->rescue_count.p,
-                    ctx->n_sms, ctx->mod_hits));
+                    ctx->n_sms, ctx->mod_hits, order));
     CK(copy_back(ctx, p_out, po, 24 * N, on_device));
     CK(copy_back(ctx, c_out, co, 84 * N, on_device));
     CK(copy_back(ctx, chi2_out, xo, 4 * N, on_device));

@@ -172,14 +172,20 @@ cudaError_t fit_static_scratch_address(void** base);
 cudaError_t launch_fit(cudaStream_t st, const DevGeom* g, DevParams P, const float4* pay, int64_t n_hits, int n,
                        int max_steps, const int* layers, const int* hits, const float* p0, const float* c0,
                        float* p_out, float* c_out, float* chi2_out, int* status_out, unsigned long long* counters,
-                       int* rescue_list, int* rescue_count, int n_sms, bool modular = false);
+                       int* rescue_list, int* rescue_count, int n_sms, bool modular = false,
+                       const int* order = nullptr);
+// Order in which a large batch's tracks are fitted (the FP32 kernels' `order`): scratch of
+// fit_order_bytes, 0 where the batch is fitted in its own order.
+size_t fit_order_bytes(int n, int max_steps);
+cudaError_t launch_fit_order(cudaStream_t st, const DevGeom* g, int n, int max_steps, const int* layers, void* scratch,
+                             const int** order);
 // Backward fit (Sec. 2.2) of n tracks listed in forward order from their state on the last
 // listed layer (covariance scaled by cov_scale); FP64 refit of tracks above kappa_fp64.
 cudaError_t launch_bkfit(cudaStream_t st, const DevGeom* g, DevParams P, const float4* pay, int64_t n_hits, int n,
                          int max_steps, const int* layers, const int* hits, const float* p_start, const float* c_start,
                          float cov_scale, float* p_out, float* c_out, float* chi2_out, int* status_out,
                          unsigned long long* counters, int* rescue_list, int* rescue_count, int n_sms,
-                         bool modular = false);
+                         bool modular = false, const int* order = nullptr);
 // Seed cleaning (mode 0) and quality filter + duplicate removal (mode 1) over n rows of `width`
 // hit ids; scratch holds clean_scratch_ints(n, width, n_hits) ints; keep gets 0/1 per row.
 size_t clean_scratch_ints(int n, int width, int64_t n_hits);

@@ -131,7 +131,8 @@ __global__ void __launch_bounds__(kThreads) k_bkfit(const DevGeom* __restrict__ 
                                                     float* __restrict__ p_out, float* __restrict__ c_out,
                                                     float* __restrict__ chi2_out, int* __restrict__ status_out,
                                                     unsigned long long* counters, int* rescue_list, int* rescue_count,
-                                                    const int* __restrict__ list, const int* __restrict__ count) {
+                                                    const int* __restrict__ list, const int* __restrict__ count,
+                                                    const int* __restrict__ order) {
     __shared__ DevGeom g;
     load_geom(gp, g);
     const int cnt = list ? *count : n;
@@ -140,7 +141,7 @@ __global__ void __launch_bounds__(kThreads) k_bkfit(const DevGeom* __restrict__ 
     // a list is dealt out to the SMs one by one, like every FP64 redo (k_fit.cu)
     const int first = list ? blockIdx.x + gridDim.x * threadIdx.x : blockIdx.x * blockDim.x + threadIdx.x;
     for (int r = first; r < cnt; r += gridDim.x * blockDim.x) {
-        const int i = list ? list[r] : r;
+        const int i = list ? list[r] : order ? order[r] : r;
         StateT<F> t;
         F sum;
         float kmax;
@@ -174,7 +175,8 @@ __global__ void __launch_bounds__(kThreads) k_bkfit(const DevGeom* __restrict__ 
 cudaError_t launch_bkfit(cudaStream_t st, const DevGeom* g, DevParams P, const float4* pay, int64_t n_hits, int n,
                          int max_steps, const int* layers, const int* hits, const float* p_start, const float* c_start,
                          float cov_scale, float* p_out, float* c_out, float* chi2_out, int* status_out,
-                         unsigned long long* counters, int* rescue_list, int* rescue_count, int n_sms, bool modular) {
+                         unsigned long long* counters, int* rescue_list, int* rescue_count, int n_sms, bool modular,
+                         const int* order) {
     if (n == 0) return cudaSuccess;
     const int blocks = (n + kThreads - 1) / kThreads;
     auto fit64 = modular ? k_bkfit<double, true> : k_bkfit<double, false>;
@@ -182,17 +184,17 @@ cudaError_t launch_bkfit(cudaStream_t st, const DevGeom* g, DevParams P, const f
     if (P.precision == MKGB_FP64) {
         fit64<<<blocks, kThreads, 0, st>>>(g, P, pay, n_hits, n, max_steps, layers, hits, p_start, c_start,
                                                      cov_scale, p_out, c_out, chi2_out, status_out, counters,
-                                                     nullptr, nullptr, nullptr, nullptr);
+                                                     nullptr, nullptr, nullptr, nullptr, nullptr);
         return cudaGetLastError();
     }
     fit32<<<blocks, kThreads, 0, st>>>(g, P, pay, n_hits, n, max_steps, layers, hits, p_start, c_start,
                                                 cov_scale, p_out, c_out, chi2_out, status_out, counters, rescue_list,
-                                                rescue_count, nullptr, nullptr);
+                                                rescue_count, nullptr, nullptr, order);
     if (P.kappa_fp64 > 0.0f && rescue_list) {
         const int rb = n < 2 * n_sms ? n : 2 * n_sms;
         fit64<<<rb, kThreads, 0, st>>>(g, P, pay, n_hits, n, max_steps, layers, hits, p_start, c_start,
                                                  cov_scale, p_out, c_out, chi2_out, status_out, counters, nullptr,
-                                                 nullptr, rescue_list, rescue_count);
+                                                 nullptr, rescue_list, rescue_count, nullptr);
     }
     return cudaGetLastError();
 }

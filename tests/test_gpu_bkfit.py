@@ -170,3 +170,25 @@ def test_fits_with_outlier_rejection_match_oracle(lib):
     sw[[i for i, _ in swaps]] = True
     ok = (rf["status"] == 0) & (ref["status"] == 0)
     assert np.mean((ref["nupd"] - rf["nupd"])[ok & sw] == 1) > 0.9
+
+
+@pytest.mark.parametrize("n", [1 << 16, (1 << 16) + 77])
+def test_fit_order_of_large_batches_changes_nothing(lib, n):
+    """Batches from 65,536 tracks on are fitted in the order of their length and layer kinds: every
+    track's results are the same bits as in a small batch, forwards and backwards; empty and
+    single-layer lists, lists longer than the others' and bad layer numbers among them."""
+    from types import SimpleNamespace
+    g, batch = _workload("phase2_small")
+    params = S.default_params()
+    fi = pipeline.fit_inputs(batch)
+    fi.layers[0], fi.hits[0] = -1, -1
+    fi.layers[1, 1:] = -1
+    fi.layers[2, 2] = g.n_layers
+    _, _, f0, b0 = _forward_then_backward(g, batch, params, fi)
+    rows = np.random.default_rng(n).integers(0, fi.layers.shape[0], n)
+    pick = lambda a: np.ascontiguousarray(a[rows])
+    big = SimpleNamespace(layers=pick(fi.layers), hits=pick(fi.hits), p0=pick(fi.p0), c0=pick(fi.c0))
+    _, _, f1, b1 = _forward_then_backward(g, batch, params, big)
+    for small, large in ((f0, f1), (b0, b1)):
+        for k in ("p", "c", "chi2", "status"):
+            assert np.array_equal(small[k][rows], large[k], equal_nan=True), k
