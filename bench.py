@@ -33,17 +33,18 @@ WORKLOAD = "phase2_like_{events}ev_20k_tracks_50k_noise_bestN6"
 # FP32 operations per unit of work (FMA = 2), counted by ncu's per-thread instruction counters
 # (FFMA/FFMA2/FADD/FADD2/FMUL/FMUL2 with true predicates) on the search and fit kernels for the
 # 8-event version of this workload, divided by the work counters of the same run:
-#   find: per crossed candidate-layer step, k_find's propagation with Jacobian, transport and
-#         material, window and chi2 of the window's hits (a4-a9);
-#   update: per Kalman update of the search, k_select's merge of the children and the Joseph
-#         update (a10-a11);
+#   find: per crossed candidate-layer step, the search's k_move, k_find and k_merge (a4-a11: the update
+#         with the candidate's last hit, its propagation with Jacobian, transport and material,
+#         window and chi2 of the window's hits, the choice of the children);
+#   update: 0 (a search update is part of its candidate's step);
 #   fit: per track-layer step of k_fit (a4-a9, a11 on one hit);
 #   seed_fp64, seed_fp32: per seed, the mixed-precision seed fit of every seed plus the FP64 refit
 #         of the low-|q/pT| ones (DFMA/DADD/DMUL and the FP32 forms), both kernels of one seed call.
 # Multi-function-unit work (sqrt, rsqrt, division seeds, sincos, log, atan2) is not counted.
-FLOPS = dict(find=1224.7, update=731.1, fit=1642.6, seed_fp64=1984.8, seed_fp32=1878.1)
+FLOPS = dict(find=1781.3, update=0.0, fit=1647.6, seed_fp64=1882.8, seed_fp32=1879.3)
 # the search and fit kernel sources the counts (and the DRAM traffic in profiles/) belong to
-KERNEL_SOURCES = ("paper_2312_11728_gb300/csrc/k_build.cu", "paper_2312_11728_gb300/csrc/kalman.cuh",
+KERNEL_SOURCES = ("paper_2312_11728_gb300/csrc/k_build.cu", "paper_2312_11728_gb300/csrc/launch.cuh",
+                  "paper_2312_11728_gb300/csrc/kalman.cuh",
                   "paper_2312_11728_gb300/csrc/trig.cuh", "paper_2312_11728_gb300/csrc/dual.cuh",
                   "paper_2312_11728_gb300/csrc/internal.h", "paper_2312_11728_gb300/build.py")
 
@@ -842,7 +843,7 @@ def main():
     # the same sources (null if the kernels changed since)
     traffic = None
     tr_path = os.path.join(ROOT, "profiles", "search_traffic.json")
-    if os.path.exists(tr_path) and shapes[0] < 3:   # captured on the two-kernel round
+    if os.path.exists(tr_path):
         tr = json.load(open(tr_path))
         if tr.get("sources_sha256_16") == kernel_sources_hash():
             traffic = tr["dram_bytes_per_crossed_step"] * int(bc[0])
@@ -851,9 +852,7 @@ def main():
     rf_search = roofline("search", stage["build"], build_flops(bc),
                          search_bytes(bc, n_hits, bins_total, n_seeds, g.max_plan), fp32_peak, hbm, traffic)
     rf_search.update({
-        "kernel": ("search: k_start, one fused k_round per plan step (k_rescue after it when flagged), k_finish"
-                   if shapes[0] >= 3 else
-                   "search: k_start, per plan step k_find and k_select (k_rescue after them when flagged), k_finish"),
+        "kernel": "search: k_start, per plan step k_move (and its FP64 redo), k_find and k_merge, k_finish",
         "peak_note": f"HBM {hbm:.1f} GB/s ({src} copy bandwidth); FP32 {n_sms} SMs x 128 lanes x 2 x {sm_max:.0f} MHz "
                      f"({src} max clock) = {fp32_peak:.1f} TFLOP/s; FMA probe {probe['fp32_tflops']:.1f} TFLOP/s",
         "launch": "algorithmic bytes and flops of one whole search over its CUDA-event time on the context's "
@@ -862,13 +861,13 @@ def main():
     rf_seed = roofline("seed", stage["seed"], FLOPS["seed_fp32"] * n_seeds, ALG_BYTES["seed"] * n_seeds, fp32_peak,
                        hbm, fp64_flops=FLOPS["seed_fp64"] * n_seeds, fp64_peak=probe["fp64_tflops"])
     keys_total = batch.n_events * 32 * 64
-    # hits: prep, scatter, scans; seeds: fit, key, scans, scatter; search: start, per plan step of
-    # the longest plan the fused round (or find and select) and the FP64 redo, finish; fit: FP32
-    # fit and FP64 refit
+    # hits: prep, scatter, scan; seeds: fit, FP64 redo, keys, scatter, scan; search: start, per step of
+    # the longest plan move, find and merge and (from the second on) the FP64 redo, finish and its
+    # redo; fit: FP32 fit and FP64 refit, the order's keys, scan and scatter for large batches
     redo = 1 if params["kappa_fp64"] > 0 else 0
-    per_round = (1 if shapes[0] >= 3 else 2) + redo
-    launches_per_step = ((2 + scan_launches(bins_total)) + (2 + scan_launches(keys_total)) + 2
-                         + per_round * g.max_plan + 1 + redo)
+    launches_per_step = ((2 + scan_launches(bins_total)) + (4 + scan_launches(keys_total))
+                         + 2 + 3 * g.max_plan + redo * g.max_plan
+                         + 1 + redo + (3 if n_tracks >= 65536 else 0))
     clocks = clk.summary()
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
