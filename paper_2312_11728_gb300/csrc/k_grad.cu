@@ -8,8 +8,8 @@
 // The kernels run the FP32 fit step (fit_step below) on dual numbers (dual.cuh) carrying KD
 // directional derivatives.
 //
-// Reverse sweep (the default): a plain FP32 pass (k_fit_ck) stores the input state of every step (a
-// checkpoint per layer); then (k_fit_adjoint), from the last step back to the first, the step is
+// Reverse sweep (the default, k_fit_adjoint, launched twice): a plain FP32 pass stores the input state
+// of every step (a checkpoint per layer); then, from the last step back to the first, the step is
 // redone from its checkpoint with its 34 inputs (27 state words, 6 alignment, 1 thickness scale)
 // seeded KD at a time, and the adjoint of its output (d total / d output, starting at zero after
 // the last step; the step's own chi2 enters with weight 1) is contracted with the output
@@ -40,9 +40,8 @@ __device__ __forceinline__ void load_geom(const DevGeom* __restrict__ gp, DevGeo
 
 __device__ __forceinline__ D seeded(float v, int comp, int base) {
     D r(v);
-#pragma unroll
-    for (int k = 0; k < KD; ++k)
-        if (comp - base == k) r.d[k] = 1.0f;
+    const int k = comp - base;
+    if (k >= 0 && k < KD) r.d[k] = 1.0f;
     return r;
 }
 
@@ -219,47 +218,6 @@ constexpr int kStateIn = 27, kStepIn = 34;
 // cross disks.
 constexpr int kAdjKeyLen = 64, kAdjKeyDisks = 32, kAdjKeys = kAdjKeyLen * kAdjKeyDisks;
 
-// Plain pass of the reverse sweep: one thread per track, the input of every step checkpointed.
-template <bool MOD>
-__global__ void __launch_bounds__(kThreads) k_fit_ck(
-    const DevGeom* __restrict__ gp, DevParams P, const float4* __restrict__ pay, int64_t n_hits, int n,
-    int max_steps, const int* __restrict__ layers, const int* __restrict__ hits, const float* __restrict__ p0,
-    const float* __restrict__ c0, const float* __restrict__ align, const float* __restrict__ xscale,
-    float* __restrict__ chi2_out, int4* __restrict__ trk, int* __restrict__ key_counts, float* __restrict__ ck) {
-    __shared__ DevGeom g;
-    load_geom(gp, g);
-    __syncthreads();
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const int* lrow = layers + (int64_t)i * max_steps;
-    const int* hrow = hits + (int64_t)i * max_steps;
-    int nl = 0;
-    while (nl < max_steps && lrow[nl] >= 0 && lrow[nl] < g.n_layers) ++nl;
-    State t;
-    {
-        const float* pi = p0 + 6 * (int64_t)i;
-        const float* ci = c0 + 21 * (int64_t)i;
-        t.xh = pi[0]; t.yh = pi[1]; t.zh = pi[2];
-        t.xl = 0.0f; t.yl = 0.0f; t.zl = 0.0f;
-        t.k = pi[3]; t.phi = pi[4]; t.th = pi[5];
-#pragma unroll
-        for (int q = 0; q < 21; ++q) t.c[q] = ci[q];
-    }
-    int status = 0, disks = 0;
-    float chi2v = 0.0f;
-    for (int j = 0; j < nl && status == 0; ++j) {
-        const int l = lrow[j];
-        disks += g.layers[l].kind == MKGB_DISK;
-        store_ck(ck + ((int64_t)j * n + i) * 32, t);
-        float x2 = 0.0f;
-        status = fit_step<float, MOD>(g, P, pay, n_hits, l, hrow[j], t, align + 6 * l, xscale[l], x2);
-        chi2v += x2;
-    }
-    chi2_out[i] = chi2v;
-    const int key = (kAdjKeyLen - 1 - min(status == 0 ? nl : 0, kAdjKeyLen - 1)) * kAdjKeyDisks + min(disks, kAdjKeyDisks - 1);
-    trk[i] = make_int4(nl, status, key, atomicAdd(key_counts + key, 1));
-}
-
 __global__ void __launch_bounds__(256) k_adj_order(int n, const int4* __restrict__ trk,
                                                    const int* __restrict__ key_off, int* __restrict__ order) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
@@ -279,9 +237,17 @@ __global__ void __launch_bounds__(256) k_adj_order(int n, const int4* __restrict
 // 1 to kAdjWide groups of 32 tracks per block: four make 68 passes for 8 warps (9 rounds, 94%
 // busy), one 3 rounds (71%); the launch takes the number with the fewest rounds over all blocks.
 // 100k tracks, 12 layers each, of the misaligned endcap: 23.4 ms with one thread per track; passes
-// shared by the warps 14.5, rounds started together 12.3, in order 9.5 ms; 1,001 tracks:
-// 5.77 -> 0.82 ms.  One direction per pass (KD = 1, 12 warps of 168 registers) rounds the
+// shared by the warps 14.5, rounds started together 12.3, in order 9.5, the directions seeded by index 8.9 ms; 1,001
+// tracks: 5.77 -> 0.82 ms.  One direction per pass (KD = 1, 12 warps of 168 registers) rounds the
 // derivatives differently: d/dp0 of a few ill-conditioned tracks moves by up to 1e-3.
+//
+// plain: the pass that writes the checkpoints, one thread per track, the input of every step stored;
+// trk and the keys' counts for the order are its results too.  It is a launch of the same kernel, not
+// a kernel of its own, because the compiler rounds the step's FP32 operations differently there (0.3%
+// of the tracks' first steps in the last bit), which d/dp0 of ill-conditioned tracks turns into up to
+// 1.2e-3 of its norm over a batch; in one function with the dual step its values have been the same
+// through every rearrangement of the sweep.  (255 registers instead of 119 cost it 0.1 ms of 100k
+// tracks' 8.9.)
 constexpr int kAdjWarps = 8, kAdjThreads = 32 * kAdjWarps;
 constexpr int kAdjPasses = (kStepIn + KD - 1) / KD;
 constexpr int kAdjWide = 4;   // groups of 32 tracks per block where the batch fills the device
@@ -291,8 +257,9 @@ __global__ void __launch_bounds__(kAdjThreads, 1) k_fit_adjoint(
     const DevGeom* __restrict__ gp, DevParams P, const float4* __restrict__ pay, int64_t n_hits, int n,
     int max_steps, const int* __restrict__ layers, const int* __restrict__ hits, const float* __restrict__ align,
     const float* __restrict__ xscale, float* __restrict__ chi2_out, float* __restrict__ d_p0,
-    float* __restrict__ d_align, float* __restrict__ d_xscale, int* __restrict__ status_out,
-    const int4* __restrict__ trk, const int* __restrict__ order, const float* __restrict__ ck, int groups) {
+    float* __restrict__ d_align, float* __restrict__ d_xscale, int* __restrict__ status_out, int4* trk,
+    const int* __restrict__ order, float* ck, int groups, bool plain, const float* __restrict__ p0,
+    const float* __restrict__ c0, int* key_counts) {
     __shared__ DevGeom g;
     __shared__ float acc[MKGB_MAX_LAYERS * 7];
     __shared__ int s_nl[32 * kAdjWide];   // steps to redo; 0 once a redone step has failed
@@ -305,6 +272,41 @@ __global__ void __launch_bounds__(kAdjThreads, 1) k_fit_adjoint(
     const int tracks = 32 * groups;
     load_geom(gp, g);
     for (int q = threadIdx.x; q < MKGB_MAX_LAYERS * 7; q += blockDim.x) acc[q] = 0.0f;
+    if (plain) {
+        __syncthreads();
+        const int i = blockIdx.x * blockDim.x + threadIdx.x;
+        if (i < n) {
+            const int* lrow = layers + (int64_t)i * max_steps;
+            const int* hrow = hits + (int64_t)i * max_steps;
+            int nl = 0;
+            while (nl < max_steps && lrow[nl] >= 0 && lrow[nl] < g.n_layers) ++nl;
+            State t;
+            {
+                const float* pi = p0 + 6 * (int64_t)i;
+                const float* ci = c0 + 21 * (int64_t)i;
+                t.xh = pi[0]; t.yh = pi[1]; t.zh = pi[2];
+                t.xl = 0.0f; t.yl = 0.0f; t.zl = 0.0f;
+                t.k = pi[3]; t.phi = pi[4]; t.th = pi[5];
+#pragma unroll
+                for (int q = 0; q < 21; ++q) t.c[q] = ci[q];
+            }
+            int status = 0, disks = 0;
+            float chi2v = 0.0f;
+            for (int j = 0; j < nl && status == 0; ++j) {
+                const int l = lrow[j];
+                disks += g.layers[l].kind == MKGB_DISK;
+                store_ck(ck + ((int64_t)j * n + i) * 32, t);
+                float x2 = 0.0f;
+                status = fit_step<float, MOD>(g, P, pay, n_hits, l, hrow[j], t, align + 6 * l, xscale[l], x2);
+                chi2v += x2;
+            }
+            chi2_out[i] = chi2v;
+            const int len = status == 0 ? nl : 0;
+            const int key = (kAdjKeyLen - 1 - min(len, kAdjKeyLen - 1)) * kAdjKeyDisks + min(disks, kAdjKeyDisks - 1);
+            trk[i] = make_int4(nl, status, key, atomicAdd(key_counts + key, 1));
+        }
+        return;
+    }
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     for (int64_t i0 = (int64_t)blockIdx.x * tracks; i0 < n; i0 += (int64_t)gridDim.x * tracks) {
         __syncthreads();   // the geometry and acc are set; the last tracks' adjoints are written out
@@ -424,7 +426,6 @@ cudaError_t launch_fit_grad(cudaStream_t st, const DevGeom* g, DevParams P, cons
     if (n == 0) return cudaSuccess;
     const int blocks = (n + kThreads - 1) / kThreads;
     if (ck) {
-        auto plain = modular ? k_fit_ck<true> : k_fit_ck<false>;
         auto adjoint = modular ? k_fit_adjoint<true> : k_fit_adjoint<false>;
         // after the checkpoints: per track (steps, status, key, rank), the keys' counts, the order
         int4* trk = reinterpret_cast<int4*>(ck + (size_t)32 * n * (max_steps > 0 ? max_steps : 1));
@@ -432,8 +433,9 @@ cudaError_t launch_fit_grad(cudaStream_t st, const DevGeom* g, DevParams P, cons
         int* order = key_counts + kAdjKeys + 4;
         cudaError_t e = cudaMemsetAsync(key_counts, 0, 4 * kAdjKeys, st);
         if (e != cudaSuccess) return e;
-        plain<<<blocks, kThreads, 0, st>>>(g, P, pay, n_hits, n, max_steps, layers, hits, p0, c0, align, xscale,
-                                           chi2_out, trk, key_counts, ck);
+        adjoint<<<blocks, kThreads, 0, st>>>(g, P, pay, n_hits, n, max_steps, layers, hits, align, xscale, chi2_out, d_p0,
+                                             d_align, d_xscale, status_out, trk, nullptr, ck, 1, true, p0, c0,
+                                             key_counts);
         if ((e = cudaGetLastError()) != cudaSuccess) return e;
         if ((e = exclusive_scan(st, key_counts, key_counts, kAdjKeys, nullptr)) != cudaSuccess) return e;   // one block
         k_adj_order<<<(n + 255) / 256, 256, 0, st>>>(n, trk, key_counts, order);
@@ -451,7 +453,7 @@ cudaError_t launch_fit_grad(cudaStream_t st, const DevGeom* g, DevParams P, cons
         }
         adjoint<<<need < n_sms ? need : n_sms, kAdjThreads, 2 * kStateIn * 32 * groups * sizeof(float), st>>>(
             g, P, pay, n_hits, n, max_steps, layers, hits, align, xscale, chi2_out, d_p0, d_align, d_xscale,
-            status_out, trk, order, ck, groups);
+            status_out, trk, order, ck, groups, false, nullptr, nullptr, nullptr);
         return cudaGetLastError();
     }
     auto forward = modular ? k_fit_grad<true> : k_fit_grad<false>;
