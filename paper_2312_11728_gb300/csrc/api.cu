@@ -414,6 +414,13 @@ int mkgb_load_modules(mkgb_ctx* ctx, int n_modules, const int32_t* layer, const 
         modular[l] = true;
     }
     DevGuard guard(ctx->device);
+    // the table that the loaded hits refer to is regrown and rewritten: hits are matched to the modules
+    // when they are loaded, and without a table no module hits can be
+    ctx->has_hits = false;
+    ctx->has_seeds = false;
+    ctx->mod_hits = false;
+    ctx->geom_h.mods = nullptr;
+    ctx->geom_h.n_mods = 0;
     if (n_modules > 0) {
         CK(ensure(ctx->mods_d, 32 * (size_t)n_modules));
         CK(cudaMemcpyAsync(ctx->mods_d.p, tab.data(), 32 * (size_t)n_modules, cudaMemcpyHostToDevice, ctx->stream));
@@ -421,12 +428,7 @@ int mkgb_load_modules(mkgb_ctx* ctx, int n_modules, const int32_t* layer, const 
     ctx->geom_h.mods = n_modules > 0 ? (const float4*)ctx->mods_d.p : nullptr;
     ctx->geom_h.n_mods = n_modules;
     for (int l = 0; l < ctx->n_layers; ++l) ctx->geom_h.layers[l].modular = modular[l] ? 1 : 0;
-    const int rc = upload_geometry(ctx);   // synchronises: tab may go
-    if (rc != MKGB_OK) return rc;
-    ctx->has_hits = false;   // hits are matched to the modules when they are loaded
-    ctx->has_seeds = false;
-    ctx->mod_hits = false;
-    return MKGB_OK;
+    return upload_geometry(ctx);   // synchronises: tab may go
 }
 
 int mkgb_set_params(mkgb_ctx* ctx, const mkgb_params* p) {
@@ -497,6 +499,11 @@ int load_hits_impl(mkgb_ctx* ctx, int n_events, const int64_t* seg_off, const fl
         CK(cudaEventCreateWithFlags(&ctx->ev_prep, cudaEventDisableTiming));
         CK(cudaEventCreateWithFlags(&ctx->ev_bins, cudaEventDisableTiming));
     }
+    // From here on the buffers of the hits loaded before are regrown and rewritten: a load that fails
+    // part-way (no memory, modules that do not fit) leaves no hits and no seeds, so that nothing runs
+    // on half a batch (the search follows hit ids that the binning has written).
+    ctx->has_hits = false;
+    ctx->has_seeds = false;
     // the previous call's binning must be done before its inputs and outputs are rewritten
     if (ctx->bins_pending) {
         CK(cudaStreamWaitEvent(st, ctx->ev_bins, 0));
@@ -554,7 +561,6 @@ int load_hits_impl(mkgb_ctx* ctx, int n_events, const int64_t* seg_off, const fl
                            n > 0 ? dm : nullptr, ctx->geom_h.bins_per_event, (float4*)ctx->pay.p,
                            (int4*)ctx->place.p, (int*)ctx->hit_seg.p, (int*)ctx->bins.p));
     }
-    ctx->has_hits = false;
     if (hit_module && n > 0) {   // every module id must fit its hit's layer (synchronises)
         CK(ensure(ctx->mod_bad, 16));
         CK(cudaMemsetAsync(ctx->mod_bad.p, 0, 4, st));
@@ -578,7 +584,6 @@ int load_hits_impl(mkgb_ctx* ctx, int n_events, const int64_t* seg_off, const fl
     ctx->n_events = n_events;
     ctx->n_hits = n;
     ctx->has_hits = true;
-    ctx->has_seeds = false;
     ctx->mod_hits = modular;
     return MKGB_OK;
 }
@@ -612,6 +617,7 @@ int mkgb_seed(mkgb_ctx* ctx, int n_seeds, const int32_t* seed_hits, int on_devic
     const int n = n_seeds;
     const void* sh = nullptr;
     CK(stage_in(ctx, S_A, seed_hits, 12 * (size_t)n, on_device, &sh));
+    ctx->has_seeds = false;   // the last seeds' buffers are regrown: true again once these are in order
     int rc = seed_buffers(ctx, n);
     if (rc != MKGB_OK) return rc;
     void *s6 = nullptr, *c21 = nullptr, *i3 = nullptr;
@@ -638,7 +644,7 @@ int mkgb_seed(mkgb_ctx* ctx, int n_seeds, const int32_t* seed_hits, int on_devic
 
 int mkgb_build(mkgb_ctx* ctx, const mkgb_tracks* out, int on_device) {
     if (!ctx) return MKGB_EINVAL;
-    if (!ctx->has_seeds) return fail(ctx, MKGB_ESTATE, "build before seed");
+    if (!ctx->has_hits || !ctx->has_seeds) return fail(ctx, MKGB_ESTATE, "build before seed");
     if (!out || !out->params || !out->cov || !out->chi2 || !out->score || !out->nfound || !out->nholes || !out->hits)
         return fail(ctx, MKGB_EINVAL, "null output array");
     if (out->max_plan < ctx->max_plan_len) return fail(ctx, MKGB_EINVAL, "max_plan %d < longest plan %d", out->max_plan, ctx->max_plan_len);
@@ -1129,6 +1135,8 @@ int run_host_impl(mkgb_ctx* ctx, int n_events, const int64_t* seg_off, const flo
     CK(cudaEventRecord(ctx->ev_fitin, ctx->cp_in));
 
     if (!ctx->has_params) return fail(ctx, MKGB_ESTATE, "run before set_params");
+    ctx->has_hits = false;   // the last batch's buffers are rewritten from here on (load_hits_impl)
+    ctx->has_seeds = false;
     ctx->n_events = n_events;   // sizes the seed ordering's keys
     int rc = seed_buffers(ctx, n_seeds);
     if (rc != MKGB_OK) return rc;
@@ -1250,7 +1258,7 @@ int mkgb_set_launch(mkgb_ctx* ctx, int find_shape, int select_shape, int use_gra
 
 int mkgb_autotune(mkgb_ctx* ctx, int reps, int* find_shape, int* select_shape, float* ms_out) {
     if (!ctx) return MKGB_EINVAL;
-    if (!ctx->has_seeds) return fail(ctx, MKGB_ESTATE, "autotune before seed");
+    if (!ctx->has_hits || !ctx->has_seeds) return fail(ctx, MKGB_ESTATE, "autotune before seed");
     if (reps < 1) return fail(ctx, MKGB_EINVAL, "reps %d < 1", reps);
     DevGuard guard(ctx->device);
     cudaStream_t st = ctx->stream;
