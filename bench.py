@@ -899,7 +899,8 @@ def main():
         "gpu_launches": int(launches_per_step * args.steps),
         "clocks": clocks,
         "counters": {"build": [int(x) for x in bc], "fit": [int(x) for x in fc]},
-        # rank 0's timed passes counted in chi2 evaluations and Kalman updates (search + fit)
+        # rank 0's timed passes counted in chi2 evaluations and Kalman updates (search + fit; the
+        # search's updates are the hits that its candidates took, see mkgb_counters)
         "rates_per_gpu": {"chi2_per_s": (int(bc[1]) + int(fc[1])) * args.steps / wall,
                           "updates_per_s": (int(bc[2]) + int(fc[2])) * args.steps / wall},
     }

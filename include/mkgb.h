@@ -389,8 +389,10 @@ int mkgb_update(mkgb_ctx* ctx, int n, const float* p_in, const float* c_in, cons
 
 /* Work counters of the last mkgb_build (kind 0) or mkgb_fit / mkgb_fit_backward (kind 1), after the call's stream
  * work has finished: [0] candidate-layer (build) or track-layer (fit) steps on crossed layers,
- * [1] chi2 evaluations of hits inside windows, [2] Kalman updates, [3] hits tested against a
- * window, [4] Newton iterations of the barrel crossing.  Synchronises the stream. */
+ * [1] chi2 evaluations of hits inside windows, [2] Kalman updates (build: the hits that kept candidates
+ * took, less those whose update failed; of a seed's last layer only the returned candidate's update is
+ * carried out, and the others count as done), [3] hits tested against a window, [4] Newton iterations of
+ * the barrel crossing.  Synchronises the stream. */
 int mkgb_counters(mkgb_ctx* ctx, int kind, int64_t out[5]);
 
 #ifdef __cplusplus

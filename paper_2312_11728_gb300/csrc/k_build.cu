@@ -702,6 +702,7 @@ __global__ void __launch_bounds__(TH, MINB) k_merge(BuildArgs a, int tau) {
         if ((all_live >> lane) & 1) a.w.live[nxt][s_base[0] + bl + __popc(all_live & below)] = sl;
         if (p_seed) a.w.seeds[nxt][s_base[1] + bs + __popc(ms & below)] = i;
     }
+    // a hit child that is kept counts as an update: k_move and k_finish take back the ones that fail
     add_counters(a.counters, 0, 0, c_upd, 0, 0);
 }
 
@@ -746,6 +747,7 @@ __global__ void __launch_bounds__(kThreads) k_finish(BuildArgs a) {
             }
         }
         if (fail == 0) best = r;
+        else if (fail == 1) atomicAdd(a.counters + 2, ~0ull);   // k_merge counted its update (- 1)
     }
     int* hrow = a.out.hits + (int64_t)seed * a.out.max_plan;
     int* orow = a.out.ovl ? a.out.ovl + (int64_t)seed * a.out.max_plan : nullptr;
