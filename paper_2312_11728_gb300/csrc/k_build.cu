@@ -183,8 +183,12 @@ __device__ __forceinline__ void load_geom_smem(const DevGeom* __restrict__ gp, D
     __syncthreads();
 }
 
-// Adds the threads' work counts to the call's counters, one atomic per warp and count (a thread's own
-// counts fit 32 bits: it takes a share of at most 2^31 slots and stays far below that).
+// Adds the threads' work counts to the call's counters, one atomic per warp and count.  A thread's own
+// counts are below kCountCap, so that a warp's sum fits 32 bits (64-bit counts took registers that
+// k_move and k_find do not have): a thread takes at most 2^31 slots / 9,728 threads of the smallest
+// launch, with 8 updates or a few dozen Newton iterations each; k_find, whose windows can hold any
+// number of hits, adds its counts to the call's counters whenever they reach the cap.
+constexpr int kCountCap = 1 << 26;
 __device__ __forceinline__ void add_counters(unsigned long long* counters, int c0, int c1, int c2, int c3, int c4) {
     const int c[5] = {c0, c1, c2, c3, c4};
 #pragma unroll
@@ -525,6 +529,12 @@ __global__ void __launch_bounds__(TH, MINB) k_find(BuildArgs a, int tau) {
                 lrec[kTile * kGroup] = e;
             else
                 a.w.ls_more[word_at<3>(sl, j / 2 - 1)] = e;
+        }
+        if (c_tested >= kCountCap) {   // (c_chi2 is no larger; one window adds at most its layer's hits)
+            atomicAdd(a.counters + 1, (unsigned long long)c_chi2);
+            atomicAdd(a.counters + 3, (unsigned long long)c_tested);
+            c_chi2 = 0;
+            c_tested = 0;
         }
     }
     add_counters(a.counters, 0, c_chi2, 0, c_tested, 0);
