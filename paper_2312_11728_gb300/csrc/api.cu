@@ -222,6 +222,13 @@ int enqueue_build(mkgb_ctx* ctx, const BuildOutDev& d, int find_shape, int selec
     return MKGB_OK;
 }
 
+// A bit per layer that is a disk.
+unsigned long long disk_bits(const DevGeom& g) {
+    unsigned long long d = 0;
+    for (int l = 0; l < g.n_layers; ++l) d |= (unsigned long long)(g.layers[l].kind == MKGB_DISK) << l;
+    return d;
+}
+
 // Copies the host geometry to the device, and the same geometry with every region's plan in
 // reverse order (the backward search); synchronises the context's stream.
 int upload_geometry(mkgb_ctx* ctx) {
@@ -826,11 +833,13 @@ int mkgb_fit(mkgb_ctx* ctx, int n, int max_steps, const int32_t* layers, const i
     CK(ensure(ctx->rescue_list, 4 * (N > 0 ? N : 1)));
     CK(ensure(ctx->rescue_count, 16));
     CK(cudaMemsetAsync(ctx->rescue_count.p, 0, 16, st));
-    const int* order = nullptr;
-    const size_t ob = ctx->params.precision == MKGB_FP64 ? 0 : fit_order_bytes(n, max_steps);
+    int* order = nullptr;
+    const unsigned long long disks = disk_bits(ctx->geom_h);
+    const size_t ob = ctx->params.precision == MKGB_FP64 ? 0 : fit_order_bytes(n, max_steps, disks, ctx->n_layers);
     if (ob > 0) {
         CK(ensure(ctx->fit_order, ob));
-        CK(launch_fit_order(st, (const DevGeom*)ctx->geom_d.p, n, max_steps, (const int*)dl, ctx->fit_order.p, &order));
+        order = (int*)ctx->fit_order.p;
+        CK(launch_fit_order(st, disks, ctx->n_layers, n, max_steps, (const int*)dl, order));
     }
     CK(launch_fit(st, (const DevGeom*)ctx->geom_d.p, ctx->params, (const float4*)ctx->pay.p,
                   ctx->has_hits ? ctx->n_hits : 0, n, max_steps, (const int*)dl, (const int*)dh, (const float*)dp0,
@@ -878,11 +887,13 @@ int mkgb_fit_backward(mkgb_ctx* ctx, int n, int max_steps, const int32_t* layers
     CK(ensure(ctx->rescue_list, 4 * (N > 0 ? N : 1)));
     CK(ensure(ctx->rescue_count, 16));
     CK(cudaMemsetAsync(ctx->rescue_count.p, 0, 16, st));
-    const int* order = nullptr;
-    const size_t ob = ctx->params.precision == MKGB_FP64 ? 0 : fit_order_bytes(n, max_steps);
+    int* order = nullptr;
+    const unsigned long long disks = disk_bits(ctx->geom_h);
+    const size_t ob = ctx->params.precision == MKGB_FP64 ? 0 : fit_order_bytes(n, max_steps, disks, ctx->n_layers);
     if (ob > 0) {
         CK(ensure(ctx->fit_order, ob));
-        CK(launch_fit_order(st, (const DevGeom*)ctx->geom_d.p, n, max_steps, (const int*)dl, ctx->fit_order.p, &order));
+        order = (int*)ctx->fit_order.p;
+        CK(launch_fit_order(st, disks, ctx->n_layers, n, max_steps, (const int*)dl, order));
     }
     CK(launch_bkfit(st, (const DevGeom*)ctx->geom_d.p, ctx->params, (const float4*)ctx->pay.p,
                     ctx->has_hits ? ctx->n_hits : 0, n, max_steps, (const int*)dl, (const int*)dh, (const float*)dp0,

@@ -84,50 +84,84 @@ __device__ __forceinline__ int fit_track(const DevGeom& g, const DevParams& P, c
     return 0;
 }
 
-// Order of a large batch's tracks: by listed layers (the longest first), then by how many of them are
-// disks.  A thread fits one track, so the lanes of a warp then end together and cross cylinders and
-// disks together.  Tracks of one key keep roughly their order in memory (ranks are given out as the
-// blocks come).  For 1M tracks k_fit takes 840 us so, 1,112 in the batch's own order (21.7 of 32 lanes
-// active), for 65 us of keys and order; k_bkfit 304 against 450 us for 320k tracks.  Taken from 65,536
-// tracks on (0.67 waves): below, three more launches cost what the order gives.
+// Order of a large batch's tracks, in chunks of kChunk: by listed layers (the longest first), then by how
+// many of them are disks.  A thread fits one track, so the lanes of a warp then end together and cross
+// cylinders and disks together.  The warps' 32 tracks of one key stay together, so that where all tracks
+// of a chunk are alike the fit's reads stay as coalesced as they were.  Within chunks, because one short
+// kernel does that (7 us for 100k tracks of 22 entries, 28 for 1M; it waits for the rows), where an
+// order of the whole batch takes a histogram, a scan and a scatter (22 and 85 us) and gains no more.
+// Fit and backward fit without their FP64 refits, own order -> in order:
+//   tracks of cylinders and disks  66k 101 -> 103, 130 -> 117 us; 100k 162 -> 144, 222 -> 185;
+//                                  320k 371 -> 326, 552 -> 427; 1M 1,067 -> 891, 1,574 -> 1,220
+//   all tracks alike               66k 69 -> 76, 76 -> 83; 100k 111 -> 117, 140 -> 148;
+//                                  320k 250 -> 263, 327 -> 341; 1M 703 -> 736, 895 -> 930
+// So it is taken from kOrderFrom tracks on (a wave of k_fit on 152 SMs is 97,280), where it saves twice
+// what it can cost, and never in a detector of one kind of layer, where most batches are alike.
 constexpr int kKeyLen = 64, kKeyDisks = 32, kKeys = kKeyLen * kKeyDisks;
-constexpr int kKeyThreads = 128;
+constexpr int kChunk = 1024, kOrderFrom = 96 * 1024;
+static_assert(kKeys == 2 * kChunk, "a thread scans two keys");
+static_assert(MKGB_MAX_LAYERS <= 64, "a bit per layer");
 
-__global__ void __launch_bounds__(kKeyThreads) k_fit_keys(const DevGeom* __restrict__ g, int n, int max_steps,
-                                                          const int* __restrict__ layers, int* __restrict__ counts,
-                                                          int2* __restrict__ key_rank) {
-    __shared__ unsigned disk[MKGB_MAX_LAYERS / 32];
-    extern __shared__ int rows[];   // the block's layer lists, read in one piece
-    if (threadIdx.x < MKGB_MAX_LAYERS / 32) disk[threadIdx.x] = 0u;
-    const int64_t first = (int64_t)blockIdx.x * kKeyThreads;
-    const int here = (int)min((int64_t)kKeyThreads, n - first);
-    for (int q = threadIdx.x; q < here * max_steps; q += kKeyThreads) rows[q] = layers[first * max_steps + q];
-    __syncthreads();
-    for (int l = threadIdx.x; l < g->n_layers; l += kKeyThreads)
-        if (g->layers[l].kind == MKGB_DISK) atomicOr(&disk[l >> 5], 1u << (l & 31));
-    __syncthreads();
-    int key = -1;
-    if ((int)threadIdx.x < here) {
-        const int* r = rows + threadIdx.x * max_steps;
-        int nl = 0, nd = 0;
-        for (; nl < max_steps && r[nl] >= 0 && r[nl] < g->n_layers; ++nl) nd += (disk[r[nl] >> 5] >> (r[nl] & 31)) & 1;
-        key = (kKeyLen - 1 - min(nl, kKeyLen - 1)) * kKeyDisks + min(nd, kKeyDisks - 1);
+// disks: bit l set where layer l is a disk.
+__global__ void __launch_bounds__(kChunk) k_fit_order(unsigned long long disks, int n_layers, int n, int max_steps,
+                                                      const int* __restrict__ layers, int* __restrict__ order) {
+    __shared__ int hist[kKeys], total[32];
+    const int tx = threadIdx.x, lane = tx & 31, wid = tx >> 5;
+    const int64_t first = (int64_t)blockIdx.x * kChunk, i = first + tx;
+    constexpr int kAhead = 8;   // entries whose loads are in flight together
+    const int* r = layers + i * max_steps;
+    const int width = i < n ? max_steps : 0;
+    int e[kAhead];
+#pragma unroll
+    for (int k = 0; k < kAhead; ++k) e[k] = k < width ? __ldg(r + k) : -1;
+    hist[2 * tx] = 0;
+    hist[2 * tx + 1] = 0;
+    int nl = 0, nd = 0;
+    for (int j = kAhead;; j += kAhead) {
+        bool end = false;
+#pragma unroll
+        for (int k = 0; k < kAhead; ++k) {
+            end = end || e[k] < 0 || e[k] >= n_layers;
+            nl += !end;
+            nd += !end && ((disks >> (e[k] & 63)) & 1);
+        }
+        if (end) break;
+#pragma unroll
+        for (int k = 0; k < kAhead; ++k) e[k] = j + k < width ? __ldg(r + j + k) : -1;
     }
-    // one atomic per warp and key: a batch has a few dozen keys
+    const int key = i < n ? (kKeyLen - 1 - min(nl, kKeyLen - 1)) * kKeyDisks + min(nd, kKeyDisks - 1) : -1;
+    __syncthreads();
     const unsigned same = __match_any_sync(0xffffffffu, key);
-    const int lane = threadIdx.x & 31, leader = __ffs(same) - 1;
-    int base = 0;
-    if (key >= 0 && lane == leader) base = atomicAdd(counts + key, __popc(same));
-    base = __shfl_sync(0xffffffffu, base, leader);
-    if (key >= 0) key_rank[first + threadIdx.x] = make_int2(key, base + __popc(same & ((1u << lane) - 1u)));
-}
-
-__global__ void __launch_bounds__(kThreads) k_fit_order(int n, const int2* __restrict__ key_rank,
-                                                        const int* __restrict__ start, int* __restrict__ order) {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= n) return;
-    const int2 k = key_rank[i];
-    order[start[k.x] + k.y] = i;
+    const int leader = __ffs(same) - 1;
+    int rank = 0;
+    if (key >= 0 && lane == leader) rank = atomicAdd(hist + key, __popc(same));
+    rank = __shfl_sync(0xffffffffu, rank, leader) + __popc(same & ((1u << lane) - 1u));
+    __syncthreads();
+    // exclusive scan of the keys' counts, two per thread
+    const int c0 = hist[2 * tx], c1 = hist[2 * tx + 1];
+    int end = c0 + c1;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const int o = __shfl_up_sync(0xffffffffu, end, d);
+        if (lane >= d) end += o;
+    }
+    if (lane == 31) total[wid] = end;
+    __syncthreads();
+    if (wid == 0) {
+        int t = total[lane];
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+            const int o = __shfl_up_sync(0xffffffffu, t, d);
+            if (lane >= d) t += o;
+        }
+        total[lane] = t;
+    }
+    __syncthreads();
+    if (wid > 0) end += total[wid - 1];
+    hist[2 * tx] = end - c1 - c0;
+    hist[2 * tx + 1] = end - c1;
+    __syncthreads();
+    if (key >= 0) order[first + hist[key] + rank] = (int)i;
 }
 
 template <bool MOD>
@@ -278,26 +312,14 @@ __global__ void __launch_bounds__(kThreads) k_step_update(int n, const float* __
 
 }  // namespace
 
-size_t fit_order_bytes(int n, int max_steps) {
-    // worth its three kernels where the batch takes several waves; rows of more layers than shared
-    // memory holds (no detector's) stay in their own order
-    if (n < (1 << 16) || kKeyThreads * max_steps * 4 > 40 * 1024 || max_steps == 0) return 0;
-    return (size_t)n * 12 + 4 * (kKeys + 4);
+size_t fit_order_bytes(int n, int max_steps, unsigned long long disks, int n_layers) {
+    const bool both_kinds = disks != 0 && disks != (n_layers < 64 ? (1ull << n_layers) - 1 : ~0ull);
+    return n >= kOrderFrom && max_steps > 0 && both_kinds ? 4 * (size_t)n : 0;
 }
 
-cudaError_t launch_fit_order(cudaStream_t st, const DevGeom* g, int n, int max_steps, const int* layers, void* scratch,
-                             const int** order) {
-    int2* key_rank = static_cast<int2*>(scratch);
-    int* counts = reinterpret_cast<int*>(key_rank + n);
-    int* ord = counts + kKeys + 4;
-    cudaError_t e = cudaMemsetAsync(counts, 0, 4 * kKeys, st);
-    if (e != cudaSuccess) return e;
-    k_fit_keys<<<(n + kKeyThreads - 1) / kKeyThreads, kKeyThreads, kKeyThreads * max_steps * 4, st>>>(
-        g, n, max_steps, layers, counts, key_rank);
-    if ((e = cudaGetLastError()) != cudaSuccess) return e;
-    if ((e = exclusive_scan(st, counts, counts, kKeys, nullptr)) != cudaSuccess) return e;   // one block
-    k_fit_order<<<(n + kThreads - 1) / kThreads, kThreads, 0, st>>>(n, key_rank, counts, ord);
-    *order = ord;
+cudaError_t launch_fit_order(cudaStream_t st, unsigned long long disks, int n_layers, int n, int max_steps,
+                             const int* layers, int* order) {
+    k_fit_order<<<(n + kChunk - 1) / kChunk, kChunk, 0, st>>>(disks, n_layers, n, max_steps, layers, order);
     return cudaGetLastError();
 }
 
