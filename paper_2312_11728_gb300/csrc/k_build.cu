@@ -878,6 +878,11 @@ __global__ void __launch_bounds__(kThreads) k_bw_seed(const DevGeom* __restrict_
 // Launch shapes of the round kernels (threads per block, minimum resident blocks per SM), one of
 // which the autotuner picks: k_move x k_find.  The resident grid of each shape is computed once,
 // before any capture.
+//
+// The FP64 redo: one block of 256 threads per SM.  Its list is empty or short at the default kappa_fp64
+// (a block of 64 or of 512 threads does it as well), but a caller may lower that until every child is on
+// it: searches of 160,000 seeds at 2^24, 2^8 and 1 took 2.38, 7.4 and 37.6 ms with blocks of 64 threads,
+// 2.37, 3.7 and 9.6 with 256, 2.39, 3.7 and 9.4 with 512.
 template <class F, int TH, int MINB, bool BWD, bool REDO = false> struct MoveShape {
     static int grid(int n_sms) {
         static int g = 0;
@@ -951,7 +956,7 @@ cudaError_t launch_rounds(cudaStream_t st, const BuildArgs& a, int n, int max_pl
     for (int tau = 0; tau < max_plan_len; ++tau) {
         with_move_shape<F, BWD>(find_shape, [&](auto s) { decltype(s)::launch(st, a, tau, n_sms); });
         if constexpr (sizeof(F) == 4) {
-            if (a.P.kappa_fp64 > 0.0f && tau > 0) MoveShape<F, 64, 1, BWD, true>::launch(st, a, tau, n_sms);
+            if (a.P.kappa_fp64 > 0.0f && tau > 0) MoveShape<F, 256, 1, BWD, true>::launch(st, a, tau, n_sms);
         }
         with_find_shape<F>(select_shape, [&](auto s) { decltype(s)::launch(st, a, tau, n_sms); });
         MergeShape<F, 256, 4>::launch(st, a, tau, n_sms);
