@@ -890,7 +890,7 @@ template <class F, int TH, int MINB, bool BWD, bool REDO = false> struct MoveSha
         return g;
     }
     static void launch(cudaStream_t st, const BuildArgs& a, int tau, int n_sms) {
-        launch_next(k_move<F, TH, MINB, BWD, REDO>, REDO ? n_sms : grid(n_sms), TH, st, a, tau);
+        launch_next(k_move<F, TH, MINB, BWD, REDO>, REDO ? n_sms : grid(n_sms), TH, st, true, a, tau);
     }
 };
 template <class F, int TH, int MINB> struct FindShape {
@@ -900,7 +900,7 @@ template <class F, int TH, int MINB> struct FindShape {
         return g;
     }
     static void launch(cudaStream_t st, const BuildArgs& a, int tau, int n_sms) {
-        launch_next(k_find<F, TH, MINB>, grid(n_sms), TH, st, a, tau);
+        launch_next(k_find<F, TH, MINB>, grid(n_sms), TH, st, true, a, tau);
     }
 };
 template <class F, int TH, int MINB> struct MergeShape {
@@ -910,7 +910,7 @@ template <class F, int TH, int MINB> struct MergeShape {
         return g;
     }
     static void launch(cudaStream_t st, const BuildArgs& a, int tau, int n_sms) {
-        launch_next(k_merge<F, TH, MINB>, grid(n_sms), TH, st, a, tau);
+        launch_next(k_merge<F, TH, MINB>, grid(n_sms), TH, st, true, a, tau);
     }
 };
 
@@ -961,9 +961,9 @@ cudaError_t launch_rounds(cudaStream_t st, const BuildArgs& a, int n, int max_pl
         with_find_shape<F>(select_shape, [&](auto s) { decltype(s)::launch(st, a, tau, n_sms); });
         MergeShape<F, 256, 4>::launch(st, a, tau, n_sms);
     }
-    launch_next(k_finish<F, false>, nb, kThreads, st, a);
+    launch_next(k_finish<F, false>, nb, kThreads, st, true, a);
     if constexpr (sizeof(F) == 4) {
-        if (a.P.kappa_fp64 > 0.0f) launch_next(k_finish<F, true>, nb, kThreads, st, a);
+        if (a.P.kappa_fp64 > 0.0f) launch_next(k_finish<F, true>, nb, kThreads, st, true, a);
     }
     return cudaGetLastError();
 }

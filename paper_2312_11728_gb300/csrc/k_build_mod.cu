@@ -835,8 +835,8 @@ template <class F, int TH, int MINB, bool BWD = false> struct FindShape {
         if (!g) g = resident_grid((const void*)k_find<F, TH, MINB, BWD>, n_sms, TH);
         return g;
     }
-    static void launch(cudaStream_t st, const BuildArgs& a, int tau, int n_sms) {
-        launch_next(k_find<F, TH, MINB, BWD>, grid(n_sms), TH, st, a, tau);
+    static void launch(cudaStream_t st, const BuildArgs& a, int tau, int n_sms, bool early) {
+        launch_next(k_find<F, TH, MINB, BWD>, grid(n_sms), TH, st, early, a, tau);
     }
 };
 template <class F, int TH, int MINB> struct SelectShape {
@@ -845,19 +845,26 @@ template <class F, int TH, int MINB> struct SelectShape {
         if (!g) g = resident_grid((const void*)k_select<F, TH, MINB>, n_sms, TH);
         return g;
     }
-    static void launch(cudaStream_t st, const BuildArgs& a, int tau, int n_sms) {
-        launch_next(k_select<F, TH, MINB>, grid(n_sms), TH, st, a, tau);
+    static void launch(cudaStream_t st, const BuildArgs& a, int tau, int n_sms, bool early) {
+        launch_next(k_select<F, TH, MINB>, grid(n_sms), TH, st, early, a, tau);
     }
 };
 
-// find_shape 0-2 (and 3-5 again): blocks of 64 x 8, 128 x 1 (the default), 256 x 1; the backward search
-// takes 128 x 1.  With 128 registers (64 x 8) the call for a module hit spills more than its own stack:
-// 0.89 ms for the search of 12,000 seeds and 2.34 for 60,000, against 0.77 and 2.30 with all 197.
-template <class F, bool BWD, class Do> void with_find_shape(int shape, Do&& f) {
+// From this many seeds on a round's kernels start behind one another and k_find runs 64 x 8 by default.
+// With 197 registers (128 x 1) it has no spills beside the stack of the call for a module hit, with 128
+// (64 x 8) twice the warps; blocks that start early take room that the large rounds of 64 x 8 use (their
+// waiting blocks hold registers and shared memory).  Search, 128 x 1 early / 64 x 8 early / 64 x 8:
+// 41,169 seeds 1.98 / 2.03 / 2.11 ms; 123,507 4.82 / 4.80 / 4.81; 205,845 7.50 / 7.53 / 7.40; 329,352
+// 11.47 / 11.70 / 11.23; 494,028 16.74 / 16.88 / 16.29.
+constexpr int kLargeFrom = 1 << 17;
+
+// find_shape 0-2 (and 3-5 again): blocks of 64 x 8; 128 x 1, or from kLargeFrom seeds on 64 x 8 (the
+// default); 256 x 1.  The backward search takes 128 x 1, the FP64 search 128 x 1 by default.
+template <class F, bool BWD, class Do> void with_find_shape(int shape, int n, Do&& f) {
     if constexpr (BWD) {
         f(FindShape<F, 128, 1, true>());
     } else {
-        switch (shape % 3) {
+        switch (shape % 3 == 1 && sizeof(F) == 4 && n >= kLargeFrom ? 0 : shape % 3) {
             case 0: f(FindShape<F, 64, 8>()); break;
             case 2: f(FindShape<F, 256, 1>()); break;
             default: f(FindShape<F, 128, 1>()); break;
@@ -878,18 +885,19 @@ template <class F, bool BWD> cudaError_t launch_rounds(cudaStream_t st, const Bu
     if (e != cudaSuccess) return e;
     const int n = a.S.n, nb = (n + kThreads - 1) / kThreads;
     k_start<F><<<nb, kThreads, 0, st>>>(a);
+    const bool early = n < kLargeFrom;
     for (int tau = 0; tau < max_plan_len; ++tau) {
-        with_find_shape<F, BWD>(find_shape, [&](auto s) { decltype(s)::launch(st, a, tau, n_sms); });
-        with_select_shape<F>(select_shape, [&](auto s) { decltype(s)::launch(st, a, tau, n_sms); });
-        if (sizeof(F) == 4 && a.P.kappa_fp64 > 0.0f) launch_next(k_rescue, n_sms, kThreads, st, a, tau);
+        with_find_shape<F, BWD>(find_shape, n, [&](auto s) { decltype(s)::launch(st, a, tau, n_sms, early); });
+        with_select_shape<F>(select_shape, [&](auto s) { decltype(s)::launch(st, a, tau, n_sms, early); });
+        if (sizeof(F) == 4 && a.P.kappa_fp64 > 0.0f) launch_next(k_rescue, n_sms, kThreads, st, early, a, tau);
     }
-    launch_next(k_finish<F>, (n * kGroup + kThreads - 1) / kThreads, kThreads, st, a);
+    launch_next(k_finish<F>, (n * kGroup + kThreads - 1) / kThreads, kThreads, st, early, a);
     return cudaGetLastError();
 }
 
 template <class F, bool BWD> void prime_shapes(int n_sms) {
     for (int q = 0; q < 3; ++q) {
-        with_find_shape<F, BWD>(q, [&](auto s) { decltype(s)::grid(n_sms); });
+        with_find_shape<F, BWD>(q, 0, [&](auto s) { decltype(s)::grid(n_sms); });
         with_select_shape<F>(q, [&](auto s) { decltype(s)::grid(n_sms); });
     }
 }

@@ -13,9 +13,10 @@ namespace mk {
 __device__ __forceinline__ void next_kernel_may_start() { cudaTriggerProgrammaticLaunchCompletion(); }
 __device__ __forceinline__ void wait_for_last_kernel() { cudaGridDependencySynchronize(); }
 
-// Launch of a kernel of the chain behind its predecessor on st (not the first one).
+// Launch of a kernel of the chain behind its predecessor on st (not the first one).  early: before the
+// predecessor has ended, as above; else behind it.
 template <class... Args>
-void launch_next(void (*kernel)(Args...), int grid, int threads, cudaStream_t st, Args... args) {
+void launch_next(void (*kernel)(Args...), int grid, int threads, cudaStream_t st, bool early, Args... args) {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(threads);
@@ -24,7 +25,7 @@ void launch_next(void (*kernel)(Args...), int grid, int threads, cudaStream_t st
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr.val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = &attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = early ? 1 : 0;
     cudaLaunchKernelEx(&cfg, kernel, args...);
 }
 
