@@ -459,7 +459,6 @@ def measure_modular(mod, params, shapes, stream, local, dist):
     fi = pipeline.fit_inputs(batch)
     dev = lambda a: torch.from_numpy(np.ascontiguousarray(a)).to(f"cuda:{local}")
     ctx = pipeline.make_context(g, params, device=local, stream=stream)
-    ctx.set_launch(shapes[0], shapes[1])
     xyz, cov, hm, seeds = dev(batch.hit_xyz), dev(batch.hit_cov), dev(batch.hit_mod), dev(batch.seed_hits)
     n, nt = int(batch.seed_hits.shape[0]), int(fi.layers.shape[0])
     out = mkgb.alloc_tracks(n, g.max_plan, device=f"cuda:{local}", ovl=True)
@@ -469,6 +468,8 @@ def measure_modular(mod, params, shapes, stream, local, dist):
     res = {"events": int(batch.n_events), "seeds": n, "tracks": nt, "modules": int(g.modules.c.shape[0]),
            "modular_layers": sorted(int(l) for l in g.modules.grid)}
     for label, hmod in (("planes", hm), ("cylinders_only", None)):
+        # the shapes were tuned on hits without modules, whose search has other kernels
+        ctx.set_launch(*((1, 0) if hmod is not None else shapes[:2]))
         ctx.load_hits(batch.n_events, batch.hit_off, xyz, cov, hit_module=hmod)
         ctx.seed(seeds)
         ctx.build(out)

@@ -295,6 +295,10 @@ int mkgb_run_modular(mkgb_ctx* ctx, int n_events, const int64_t* seg_off, const 
  * and chi2; the merge per seed).  find_shape 0..5 picks the blocks of the first: 128, 128, 256, 64,
  * 64 or 128 threads with 5, 4, 2, 8, 10 or 3 of them resident per SM; select_shape 0..2 those of
  * the second: 128, 64 or 128 threads with 6, 12 or 8.  (1, 0) is the default.
+ * With module hits loaded (mkgb_load_hits_modular) a round runs as two kernels (propagation, window
+ * and chi2; merge and update) and the same numbers pick theirs: find_shape 0, 1, 2 (3, 4, 5 again)
+ * blocks of 64, 128 or 256 threads with at least 8, 1 or 1 resident per SM (1, the default: 64 with 8
+ * from 131,072 seeds on); select_shape 0, 1, 2 128, 64 or 256 threads with 5, 10 or 2.
  * Each kernel launches as many blocks as stay resident on the device.  use_graph = 1 (the
  * default) records the launches of one search as a CUDA graph on the first call and replays it
  * while the arguments, shapes and stream stay the same (a change re-records); the graph is used
@@ -306,7 +310,7 @@ int mkgb_set_launch(mkgb_ctx* ctx, int find_shape, int select_shape, int use_gra
 
 /* Autotuner of the search launch shapes (library service, no counterpart in the paper): runs
  * the search over the seeds loaded now (mkgb_seed) once per launch configuration (the 6 x 3
- * shapes of mkgb_set_launch), each warmed once and then timed
+ * shapes of mkgb_set_launch, 3 x 3 with module hits), each warmed once and then timed
  * reps times with CUDA events on the context's stream, keeps the fastest as the context's
  * shapes (mkgb_set_launch) and writes it to find_shape / select_shape (may be NULL) and its mean
  * time per search to ms_out (may be NULL).  The outputs of these searches go to the library's

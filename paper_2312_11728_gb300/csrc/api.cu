@@ -1292,7 +1292,8 @@ int mkgb_autotune(mkgb_ctx* ctx, int reps, int* find_shape, int* select_shape, f
     }
     int best_f = ctx->find_shape, best_s = ctx->select_shape, rc = MKGB_OK;
     float best = -1.0f;
-    for (int f = 0; f < 6 && rc == MKGB_OK; ++f)
+    const int n_find = ctx->mod_hits ? 3 : 6;   // with module hits shapes 3 to 5 are 0 to 2 again
+    for (int f = 0; f < n_find && rc == MKGB_OK; ++f)
         for (int s = 0; s < 3 && rc == MKGB_OK; ++s) {
             rc = enqueue_build(ctx, d, f, s);   // warm-up (and the graph's recording)
             if (rc == MKGB_OK) cudaEventRecord(e0, st);

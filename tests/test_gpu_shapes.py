@@ -38,6 +38,8 @@ def test_every_pair_of_shapes(event):
             got = _search(g, ctx, b.seed_hits)
             for k in ref:
                 assert np.array_equal(got[k], ref[k]), (f, s, k)
+    best = ctx.autotune(1)
+    assert best[0] < (3 if kind == "modules" else 6)
     ctx.set_launch(1, 0)
 
 
