@@ -165,7 +165,7 @@ __global__ void __launch_bounds__(kChunk) k_fit_order(unsigned long long disks, 
 }
 
 template <bool MOD>
-__global__ void __launch_bounds__(kThreads, MOD ? 1 : 5) k_fit(const DevGeom* __restrict__ gp, DevParams P,
+__global__ void __launch_bounds__(kThreads, MOD ? 4 : 5) k_fit(const DevGeom* __restrict__ gp, DevParams P,
                                                   const float4* __restrict__ pay, int64_t n_hits, int n, int max_steps,
                                                   const int* __restrict__ layers, const int* __restrict__ hits,
                                                   const float* __restrict__ p0, const float* __restrict__ c0,
