@@ -833,13 +833,14 @@ int mkgb_fit(mkgb_ctx* ctx, int n, int max_steps, const int32_t* layers, const i
     CK(ensure(ctx->rescue_list, 4 * (N > 0 ? N : 1)));
     CK(ensure(ctx->rescue_count, 16));
     CK(cudaMemsetAsync(ctx->rescue_count.p, 0, 16, st));
-    int* order = nullptr;
+    const int* order = nullptr;
     const unsigned long long disks = disk_bits(ctx->geom_h);
-    const size_t ob = ctx->params.precision == MKGB_FP64 ? 0 : fit_order_bytes(n, max_steps, disks, ctx->n_layers);
+    const size_t ob = ctx->params.precision == MKGB_FP64
+                          ? 0 : fit_order_bytes(n, max_steps, disks, ctx->n_layers, ctx->mod_hits);
     if (ob > 0) {
         CK(ensure(ctx->fit_order, ob));
-        order = (int*)ctx->fit_order.p;
-        CK(launch_fit_order(st, disks, ctx->n_layers, n, max_steps, (const int*)dl, order));
+        CK(launch_fit_order(st, disks, ctx->n_layers, n, max_steps, (const int*)dl, ctx->mod_hits, ctx->fit_order.p,
+                            &order));
     }
     CK(launch_fit(st, (const DevGeom*)ctx->geom_d.p, ctx->params, (const float4*)ctx->pay.p,
                   ctx->has_hits ? ctx->n_hits : 0, n, max_steps, (const int*)dl, (const int*)dh, (const float*)dp0,
@@ -887,13 +888,14 @@ int mkgb_fit_backward(mkgb_ctx* ctx, int n, int max_steps, const int32_t* layers
     CK(ensure(ctx->rescue_list, 4 * (N > 0 ? N : 1)));
     CK(ensure(ctx->rescue_count, 16));
     CK(cudaMemsetAsync(ctx->rescue_count.p, 0, 16, st));
-    int* order = nullptr;
+    const int* order = nullptr;
     const unsigned long long disks = disk_bits(ctx->geom_h);
-    const size_t ob = ctx->params.precision == MKGB_FP64 ? 0 : fit_order_bytes(n, max_steps, disks, ctx->n_layers);
+    const size_t ob = ctx->params.precision == MKGB_FP64
+                          ? 0 : fit_order_bytes(n, max_steps, disks, ctx->n_layers, ctx->mod_hits);
     if (ob > 0) {
         CK(ensure(ctx->fit_order, ob));
-        order = (int*)ctx->fit_order.p;
-        CK(launch_fit_order(st, disks, ctx->n_layers, n, max_steps, (const int*)dl, order));
+        CK(launch_fit_order(st, disks, ctx->n_layers, n, max_steps, (const int*)dl, ctx->mod_hits, ctx->fit_order.p,
+                            &order));
     }
     CK(launch_bkfit(st, (const DevGeom*)ctx->geom_d.p, ctx->params, (const float4*)ctx->pay.p,
                     ctx->has_hits ? ctx->n_hits : 0, n, max_steps, (const int*)dl, (const int*)dh, (const float*)dp0,

@@ -174,11 +174,11 @@ cudaError_t launch_fit(cudaStream_t st, const DevGeom* g, DevParams P, const flo
                        float* p_out, float* c_out, float* chi2_out, int* status_out, unsigned long long* counters,
                        int* rescue_list, int* rescue_count, int n_sms, bool modular = false,
                        const int* order = nullptr);
-// Order in which a large batch's tracks are fitted (the FP32 kernels' `order`): its bytes, 0 where the
-// batch is fitted in its own order.  disks: a bit per layer that is a disk.
-size_t fit_order_bytes(int n, int max_steps, unsigned long long disks, int n_layers);
+// Order in which a large batch's tracks are fitted (the FP32 kernels' `order`): scratch of
+// fit_order_bytes, 0 where the batch is fitted in its own order.  disks: a bit per layer that is a disk.
+size_t fit_order_bytes(int n, int max_steps, unsigned long long disks, int n_layers, bool modular);
 cudaError_t launch_fit_order(cudaStream_t st, unsigned long long disks, int n_layers, int n, int max_steps,
-                             const int* layers, int* order);
+                             const int* layers, bool modular, void* scratch, const int** order);
 // Backward fit (Sec. 2.2) of n tracks listed in forward order from their state on the last
 // listed layer (covariance scaled by cov_scale); FP64 refit of tracks above kappa_fp64.
 cudaError_t launch_bkfit(cudaStream_t st, const DevGeom* g, DevParams P, const float4* pay, int64_t n_hits, int n,

@@ -98,38 +98,65 @@ __device__ __forceinline__ int fit_track(const DevGeom& g, const DevParams& P, c
 // So it is taken from kOrderFrom tracks on (a wave of k_fit on 152 SMs is 97,280), where it saves twice
 // what it can cost, and never in a detector of one kind of layer, where most batches are alike.
 constexpr int kKeyLen = 64, kKeyDisks = 32, kKeys = kKeyLen * kKeyDisks;
-constexpr int kChunk = 1024, kOrderFrom = 96 * 1024;
+constexpr int kChunk = 1024, kOrderFrom = 96 * 1024, kOrderFromMod = 64 * 1024;
 static_assert(kKeys == 2 * kChunk, "a thread scans two keys");
 static_assert(MKGB_MAX_LAYERS <= 64, "a bit per layer");
 
-// disks: bit l set where layer l is a disk.
-__global__ void __launch_bounds__(kChunk) k_fit_order(unsigned long long disks, int n_layers, int n, int max_steps,
-                                                      const int* __restrict__ layers, int* __restrict__ order) {
-    __shared__ int hist[kKeys], total[32];
-    const int tx = threadIdx.x, lane = tx & 31, wid = tx >> 5;
-    const int64_t first = (int64_t)blockIdx.x * kChunk, i = first + tx;
+// Key of a track's layer list; disks: bit l set where layer l is a disk.
+__device__ __forceinline__ int fit_key(unsigned long long disks, int n_layers, int max_steps, const int* __restrict__ r) {
     constexpr int kAhead = 8;   // entries whose loads are in flight together
-    const int* r = layers + i * max_steps;
-    const int width = i < n ? max_steps : 0;
-    int e[kAhead];
-#pragma unroll
-    for (int k = 0; k < kAhead; ++k) e[k] = k < width ? __ldg(r + k) : -1;
-    hist[2 * tx] = 0;
-    hist[2 * tx + 1] = 0;
     int nl = 0, nd = 0;
-    for (int j = kAhead;; j += kAhead) {
-        bool end = false;
+    bool end = false;
+    for (int j = 0; !end; j += kAhead) {
+        int e[kAhead];
+#pragma unroll
+        for (int k = 0; k < kAhead; ++k) e[k] = j + k < max_steps ? __ldg(r + j + k) : -1;
 #pragma unroll
         for (int k = 0; k < kAhead; ++k) {
             end = end || e[k] < 0 || e[k] >= n_layers;
             nl += !end;
             nd += !end && ((disks >> (e[k] & 63)) & 1);
         }
-        if (end) break;
-#pragma unroll
-        for (int k = 0; k < kAhead; ++k) e[k] = j + k < width ? __ldg(r + j + k) : -1;
     }
-    const int key = i < n ? (kKeyLen - 1 - min(nl, kKeyLen - 1)) * kKeyDisks + min(nd, kKeyDisks - 1) : -1;
+    return (kKeyLen - 1 - min(nl, kKeyLen - 1)) * kKeyDisks + min(nd, kKeyDisks - 1);
+}
+
+// The order of the whole batch, with module hits: places within the keys, then (their counts scanned) the
+// order itself.  A step to a module's plane is a call that the lanes of other layers wait for, so here
+// warps of two keys cost more than three kernels do: fit and backward fit of 82,400 tracks 748 and 231 us
+// (in their own order 834 and 537), of 329,600 1,100 and 636 (1,342 and 1,822; in chunks of 16,384
+// tracks 1,199 and 832).
+__global__ void __launch_bounds__(kThreads) k_fit_keys(unsigned long long disks, int n_layers, int n, int max_steps,
+                                                       const int* __restrict__ layers, int* __restrict__ counts,
+                                                       int2* __restrict__ key_rank) {
+    const int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x;
+    const int key = i < n ? fit_key(disks, n_layers, max_steps, layers + i * max_steps) : -1;
+    // one atomic per warp and key: a batch has a few dozen keys
+    const unsigned same = __match_any_sync(0xffffffffu, key);
+    const int lane = threadIdx.x & 31, leader = __ffs(same) - 1;
+    int base = 0;
+    if (key >= 0 && lane == leader) base = atomicAdd(counts + key, __popc(same));
+    base = __shfl_sync(0xffffffffu, base, leader);
+    if (key >= 0) key_rank[i] = make_int2(key, base + __popc(same & ((1u << lane) - 1u)));
+}
+
+__global__ void __launch_bounds__(kThreads) k_fit_place(int n, const int2* __restrict__ key_rank,
+                                                        const int* __restrict__ start, int* __restrict__ order) {
+    const int i = blockIdx.x * kThreads + threadIdx.x;
+    if (i >= n) return;
+    const int2 k = key_rank[i];
+    order[start[k.x] + k.y] = i;
+}
+
+// The order within chunks.
+__global__ void __launch_bounds__(kChunk) k_fit_order(unsigned long long disks, int n_layers, int n, int max_steps,
+                                                      const int* __restrict__ layers, int* __restrict__ order) {
+    __shared__ int hist[kKeys], total[32];
+    const int tx = threadIdx.x, lane = tx & 31, wid = tx >> 5;
+    const int64_t first = (int64_t)blockIdx.x * kChunk, i = first + tx;
+    hist[2 * tx] = 0;
+    hist[2 * tx + 1] = 0;
+    const int key = i < n ? fit_key(disks, n_layers, max_steps, layers + i * max_steps) : -1;
     __syncthreads();
     const unsigned same = __match_any_sync(0xffffffffu, key);
     const int leader = __ffs(same) - 1;
@@ -312,14 +339,31 @@ __global__ void __launch_bounds__(kThreads) k_step_update(int n, const float* __
 
 }  // namespace
 
-size_t fit_order_bytes(int n, int max_steps, unsigned long long disks, int n_layers) {
+size_t fit_order_bytes(int n, int max_steps, unsigned long long disks, int n_layers, bool modular) {
     const bool both_kinds = disks != 0 && disks != (n_layers < 64 ? (1ull << n_layers) - 1 : ~0ull);
-    return n >= kOrderFrom && max_steps > 0 && both_kinds ? 4 * (size_t)n : 0;
+    if (n < (modular ? kOrderFromMod : kOrderFrom) || max_steps == 0 || !both_kinds) return 0;
+    return modular ? 12 * (size_t)n + 4 * (kKeys + 4) : 4 * (size_t)n;   // the keys and places, their counts
 }
 
 cudaError_t launch_fit_order(cudaStream_t st, unsigned long long disks, int n_layers, int n, int max_steps,
-                             const int* layers, int* order) {
-    k_fit_order<<<(n + kChunk - 1) / kChunk, kChunk, 0, st>>>(disks, n_layers, n, max_steps, layers, order);
+                             const int* layers, bool modular, void* scratch, const int** order) {
+    if (!modular) {
+        int* ord = static_cast<int*>(scratch);
+        k_fit_order<<<(n + kChunk - 1) / kChunk, kChunk, 0, st>>>(disks, n_layers, n, max_steps, layers, ord);
+        *order = ord;
+        return cudaGetLastError();
+    }
+    const int blocks = (n + kThreads - 1) / kThreads;
+    int2* key_rank = static_cast<int2*>(scratch);
+    int* counts = reinterpret_cast<int*>(key_rank + n);
+    int* ord = counts + kKeys + 4;
+    cudaError_t e = cudaMemsetAsync(counts, 0, 4 * kKeys, st);
+    if (e != cudaSuccess) return e;
+    k_fit_keys<<<blocks, kThreads, 0, st>>>(disks, n_layers, n, max_steps, layers, counts, key_rank);
+    if ((e = cudaGetLastError()) != cudaSuccess) return e;
+    if ((e = exclusive_scan(st, counts, counts, kKeys, nullptr)) != cudaSuccess) return e;   // one block
+    k_fit_place<<<blocks, kThreads, 0, st>>>(n, key_rank, counts, ord);
+    *order = ord;
     return cudaGetLastError();
 }
 

@@ -1,6 +1,6 @@
-"""Large batches are fitted in the order of their tracks' length and layer kinds, chunk by chunk: every
-track's results are the same bits as in a small batch, which keeps its own order, forwards and
-backwards."""
+"""Large batches are fitted in the order of their tracks' length and layer kinds, chunk by chunk or, with
+module hits, all together: every track's results are the same bits as in a small batch, which keeps its
+own order, forwards and backwards."""
 from types import SimpleNamespace
 
 import numpy as np
@@ -11,12 +11,13 @@ from paper_2312_11728_gb300 import mkgb, pipeline, synth as S
 
 pytestmark = pytest.mark.gpu
 
-ORDER_FROM, CHUNK = 96 * 1024, 1024   # of k_fit.cu
+ORDER_FROM, ORDER_FROM_MOD, CHUNK = 96 * 1024, 64 * 1024, 1024   # of k_fit.cu
 
 
 def _fit(g, batch, fi):
     ctx = pipeline.make_context(g, S.default_params())
-    ctx.load_hits(batch.n_events, batch.hit_off, batch.hit_xyz, batch.hit_cov)
+    ctx.load_hits(batch.n_events, batch.hit_off, batch.hit_xyz, batch.hit_cov,
+                  hit_module=None if g.modules is None else batch.hit_mod)
     n = fi.layers.shape[0]
     out = lambda: dict(p=np.zeros((n, 6), np.float32), c=np.zeros((n, 21), np.float32), x=np.zeros(n, np.float32),
                        s=np.full(n, -7, np.int32))
@@ -26,14 +27,9 @@ def _fit(g, batch, fi):
     return f, b
 
 
-@pytest.mark.parametrize("n", [ORDER_FROM - 1, ORDER_FROM, ORDER_FROM + 1, 97 * CHUNK - 1, 97 * CHUNK + 33])
-@pytest.mark.parametrize("pad", [0, 1, 40])
-def test_order_changes_no_track(n, pad):
-    """Lists without layers, of one layer, with a bad layer number and (pad) in rows wider than any track,
-    of odd and even width."""
+def _check(g, n, pad):
     B.build()
     mkgb.load_library()
-    g = S.geometry_phase2()
     batch = S.concat_events([S.simulate_event(g, 700, 11, 0, pt_sampler=S.sample_pt_phase2, eta_max=3.0, noise_total=500)],
                             g.n_layers)
     fi = pipeline.fit_inputs(batch)
@@ -50,3 +46,16 @@ def test_order_changes_no_track(n, pad):
     for a, b in zip(_fit(g, batch, small), _fit(g, batch, large)):
         for k in a:
             assert np.array_equal(a[k][rows], b[k], equal_nan=True), k
+
+
+@pytest.mark.parametrize("n", [ORDER_FROM - 1, ORDER_FROM, ORDER_FROM + 1, 97 * CHUNK - 1, 97 * CHUNK + 33])
+@pytest.mark.parametrize("pad", [0, 1, 40])
+def test_order_changes_no_track(n, pad):
+    """Lists without layers, of one layer, with a bad layer number and (pad) in rows wider than any track,
+    of odd and even width."""
+    _check(S.geometry_phase2(), n, pad)
+
+
+@pytest.mark.parametrize("n, pad", [(ORDER_FROM_MOD - 1, 0), (ORDER_FROM_MOD, 0), (ORDER_FROM_MOD + 1, 1), (70_001, 40)])
+def test_order_changes_no_track_with_modules(n, pad):
+    _check(S.geometry_phase2_modular_disks(), n, pad)
