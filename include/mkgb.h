@@ -298,7 +298,7 @@ int mkgb_run_modular(mkgb_ctx* ctx, int n_events, const int64_t* seg_off, const 
  * With module hits loaded (mkgb_load_hits_modular) a round runs as two kernels (propagation, window
  * and chi2; merge and update) and the same numbers pick theirs: find_shape 0, 1, 2 (3, 4, 5 again)
  * blocks of 64, 128 or 256 threads with at least 8, 1 or 1 resident per SM (1, the default: 64 with 8
- * from 131,072 seeds on); select_shape 0, 1, 2 128, 64 or 256 threads with 5, 10 or 2.
+ * from 114,688 seeds on); select_shape 0, 1, 2 128, 64 or 256 threads with 5, 10 or 2.
  * Each kernel launches as many blocks as stay resident on the device.  use_graph = 1 (the
  * default) records the launches of one search as a CUDA graph on the first call and replays it
  * while the arguments, shapes and stream stay the same (a change re-records); the graph is used

@@ -854,9 +854,10 @@ template <class F, int TH, int MINB> struct SelectShape {
 // With 197 registers (128 x 1) it has no spills beside the stack of the call for a module hit, with 128
 // (64 x 8) twice the warps; blocks that start early take room that the large rounds of 64 x 8 use (their
 // waiting blocks hold registers and shared memory).  Search, 128 x 1 early / 64 x 8 early / 64 x 8:
-// 41,169 seeds 1.98 / 2.03 / 2.11 ms; 123,507 4.82 / 4.80 / 4.81; 205,845 7.50 / 7.53 / 7.40; 329,352
-// 11.47 / 11.70 / 11.23; 494,028 16.74 / 16.88 / 16.29.
-constexpr int kLargeFrom = 1 << 17;
+// 41,169 seeds 1.98 / 2.03 / 2.11 ms; 82,338 3.44 / 3.46 / 3.51; 123,507 4.82 / 4.80 / 4.81 (the whole
+// pass with the fit beside it 5.79 / - / 5.72); 205,845 7.50 / 7.53 / 7.40; 329,352 11.47 / 11.70 / 11.23;
+// 494,028 16.74 / 16.88 / 16.29.
+constexpr int kLargeFrom = 7 << 14;
 
 // find_shape 0-2 (and 3-5 again): blocks of 64 x 8; 128 x 1, or from kLargeFrom seeds on 64 x 8 (the
 // default); 256 x 1.  The backward search takes 128 x 1, the FP64 search 128 x 1 by default.

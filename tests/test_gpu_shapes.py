@@ -8,7 +8,7 @@ from paper_2312_11728_gb300 import mkgb, pipeline, synth as S
 
 pytestmark = pytest.mark.gpu
 
-LARGE_FROM = 1 << 17   # of k_build_mod.cu
+LARGE_FROM = 7 << 14   # of k_build_mod.cu
 
 
 @pytest.fixture(scope="module", params=["cylinders", "modules"])
