@@ -21,9 +21,9 @@
 // merge and update by eight lanes per seed, 18.5 of 32 lanes active, states and predictions both
 // written, records one after another) took 21.6 ms for 64 Phase-2-like events (1.28M seeds, 58M
 // crossed steps) and 0.90 ms for one; one kernel for update, propagation and window 17.2 ms (its 128
-// registers also held the window's chains of loads to 16 warps); these three 15.8 and 0.65 ms:
-// k_move 7.5 ms, k_find 3.1, k_merge 4.3 of the 64 events.  k_move is bound by issue and latency
-// together (47% issue active, 28% of DRAM), k_find and k_merge by their dependent loads.
+// registers also held the window's chains of loads to 16 warps); these three 15.45 and 0.65 ms:
+// k_move 7.3 ms, k_find 3.1, k_merge 4.3 of the 64 events.  k_move is bound by issue and latency
+// together (50% issue active, 29% of DRAM), k_find and k_merge by their dependent loads.
 //
 // No kernel waits on another block; every loop is bounded by a list length, a window's bin range or
 // the Newton iteration limit.  The kernels of a search are chained by programmatic dependent
@@ -78,7 +78,6 @@ template <int N> __device__ __forceinline__ int64_t word_at(int sl, int j) {
 constexpr int kStateWords = 32, kPredWords = 28;
 static_assert(kStateWords == kSeedStateStride, "seed records are read as state records");
 template <class F> constexpr int rec_vecs() { return (int)(kStateWords * sizeof(F) / 16); }
-template <class F> constexpr size_t state_bytes() { return kStateWords * sizeof(F); }
 
 template <class F, int W> __device__ __forceinline__ void load_rec(const unsigned char* __restrict__ base, int sl, F* f) {
     using V = typename Vec16<F>::T;
@@ -545,10 +544,11 @@ __global__ void __launch_bounds__(TH, MINB) k_find(BuildArgs a, int tau) {
 // Eight lanes per seed, lane = parent slot.  Every child of the seed puts its key (score, then parent
 // slot, then place in the parent's list) into shared memory and counts the keys above its own: that
 // count is its slot among the N best, so a parent's lane writes its kept children straight from its
-// registers, with no exchange of their contents and no round per rank. 
-// 64 events: 4.3 ms (4.8 with a walk over the keys per child); eight lanes exchanging keys and contents by shuffles, a round per rank: 7.4 ms;
-// one thread per seed with its eight best in registers: 3.8 ms, but 1.3 times the whole search of one
-// event (0.86 against 0.66 ms), where the latency of a thread's serial lists counts.
+// registers, with no exchange of their contents and no round per rank.  64 registers (12 bytes spilled)
+// for 32 warps per SM.  64 events: 4.3 ms (4.8 with a walk over the keys per child); eight lanes
+// exchanging keys and contents by shuffles, a round per rank: 7.4 ms; one thread per seed with its eight
+// best in registers: 3.8 ms, but 1.3 times the whole search of one event (0.86 against 0.66 ms), where
+// the latency of a thread's serial lists counts.
 constexpr int kNoHit = 15;   // place of the child without a hit
 constexpr int kSeedKeys = kGroup * (kGroup + 1);
 __device__ __forceinline__ unsigned long long child_key(float score, int slot, int place) {
@@ -915,9 +915,10 @@ template <class F, int TH, int MINB> struct MergeShape {
 };
 
 // find_shape: k_move as blocks of 128 x 5, 128 x 4 (the default), 256 x 2, 64 x 8, 64 x 10, 128 x 3
-// (threads x resident blocks per SM): 128 registers a thread at 16 warps (no spills; 15.5 ms per
-// 64-event search), 96 at 20 (112 bytes spilled; 15.7), 138 at 12 (16.7; all with the former k_merge).  select_shape: k_find as
-// 128 x 6, 64 x 12 (80 registers), 128 x 8 (64 registers, 48 bytes spilled; 0.9 ms slower).
+// (threads x resident blocks per SM): searches of 64 events 15.91, 15.45, 15.63, 15.48, 15.92 and 16.44
+// ms (125 registers at 16 warps per SM, no spills; 96 and 116 bytes spilled at 20; 139 at 12).
+// select_shape: k_find as 128 x 6 (80 registers), 64 x 12, 128 x 8 (64 registers, 20 bytes spilled): 15.45,
+// 15.50 and 15.34 ms, one event 0.647, 0.649 and 0.670.
 template <class F, bool BWD, class Do> void with_move_shape(int shape, Do&& f) {
     if constexpr (sizeof(F) == 8) {
         f(MoveShape<F, 128, 1, BWD>());

@@ -18,12 +18,12 @@
 // k_start fills round 0 from the seed states; k_finish picks each seed's best candidate and walks
 // the trail back for its hit list (a13).
 //
-// Batches without module hits go through the rounds of k_build.cu, which are faster there (15.8
+// Batches without module hits go through the rounds of k_build.cu, which are faster there (15.45
 // against 21.6 ms for 64 events).  With module hits those rounds were 5% faster than these (0.92
-// against 0.97 ms, 12,000 seeds of two events): the step to a module's plane takes most of the time,
-// a call with its own stack either way.  But their compiled Newton loop rounds some crossings of the
-// cylinders differently, and the seeds with badly conditioned updates turn that last bit into up to
-// 2e-4 of the covariances, so these rounds stay for module hits.
+// against 0.97 ms, 12,000 seeds of two events), but their compiled FP32 step rounds a few crossings
+// differently (in which operation is not known: each kernel's contractions are the compiler's), and the
+// seeds with badly conditioned updates turn that last bit into up to 2e-4 of the covariances.  So these
+// rounds stay for module hits.
 //
 // Slot records are array-of-structures in HBM: a state is 32 words (xh, yh, zh, xl, yl, zl, k,
 // phi, theta, 21 covariance terms, theta's and phi's low parts), a prediction 28 words, a child

@@ -237,9 +237,9 @@ __global__ void __launch_bounds__(256) k_adj_order(int n, const int4* __restrict
 // 1 to kAdjWide groups of 32 tracks per block: four make 68 passes for 8 warps (9 rounds, 94%
 // busy), one 3 rounds (71%); the launch takes the number with the fewest rounds over all blocks.
 // 100k tracks, 12 layers each, of the misaligned endcap: 23.4 ms with one thread per track; passes
-// shared by the warps 14.5, rounds started together 12.3, in order 9.5, the directions seeded by index 8.9 ms; 1,001
-// tracks: 5.77 -> 0.82 ms.  One direction per pass (KD = 1, 12 warps of 168 registers) rounds the
-// derivatives differently: d/dp0 of a few ill-conditioned tracks moves by up to 1e-3.
+// shared by the warps 14.5, rounds started together 12.3, in order 9.5, the directions seeded by index
+// 8.9 ms (one direction per pass, KD = 1 with 12 warps of 168 registers, 12.1); 1,001 tracks: 5.71 ->
+// 0.74 ms.
 //
 // plain: the pass that writes the checkpoints, one thread per track, the input of every step stored;
 // trk and the keys' counts for the order are its results too.  It is a launch of the same kernel, not
