@@ -864,11 +864,11 @@ def main():
     keys_total = batch.n_events * 32 * 64
     # hits: prep, scatter, scan; seeds: fit, FP64 redo, keys, scatter, scan; search: start, per step of
     # the longest plan move, find and merge and (from the second on) the FP64 redo, finish and its
-    # redo; fit: FP32 fit and FP64 refit, the order's keys, scan and scatter for large batches
+    # redo; fit: FP32 fit and FP64 refit, and the order for large batches
     redo = 1 if params["kappa_fp64"] > 0 else 0
     launches_per_step = ((2 + scan_launches(bins_total)) + (4 + scan_launches(keys_total))
                          + 2 + 3 * g.max_plan + redo * g.max_plan
-                         + 1 + redo + (3 if n_tracks >= 65536 else 0))
+                         + 1 + redo + (1 if n_tracks >= 96 * 1024 else 0))
     clocks = clk.summary()
     line = {
         "metric": METRIC, "value": value, "unit": UNIT, "n_gpus": world, "steps": args.steps,
